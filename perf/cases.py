@@ -26,29 +26,29 @@ DEV = "cuda"
 def listed():
     return [
         # one round of a real-time loop on a small patch: pure latency
-        {"name": "one shot, d=5", "kind": "decode", "d": 5, "chi": 16, "B": 1, "noise": "table", "mixed": False},
+        {"name": "one shot d=5", "kind": "decode", "d": 5, "chi": 16, "B": 1, "noise": "table", "mixed": False},
         # a rate scan: every shot with its own depolarizing strength, no decisions kept
-        {"name": "rate scan, d=7", "kind": "decode", "d": 7, "chi": 16, "B": 262_143, "noise": "shots", "mixed": False},
+        {"name": "rate scan d=7", "kind": "decode", "d": 7, "chi": 16, "B": 262_143, "noise": "shots", "mixed": False},
         # the bench's workload: d=9, chi=32, p=0.10, all four classes, mixed precision asked for
-        {"name": "headline, d=9", "kind": "decode", "d": 9, "chi": 32, "B": 65_536, "noise": "depol", "mixed": True},
+        {"name": "headline d=9", "kind": "decode", "d": 9, "chi": 32, "B": 65_536, "noise": "depol", "mixed": True},
         # the largest distance decoded without truncation, a ragged batch
-        {"name": "untruncated, d=13", "kind": "decode", "d": 13, "chi": 64, "B": 4_099, "noise": "table",
+        {"name": "untruncated d=13", "kind": "decode", "d": 13, "chi": 64, "B": 4_099, "noise": "table",
          "mixed": False},
         # a serving batch over all untruncated distances as one graph launch
-        {"name": "mixed batch, d=3..13", "kind": "graph", "B": 131_072, "mixed": True},
+        {"name": "mixed batch d=3..13", "kind": "graph", "B": 131_072, "mixed": True},
         # large patches below threshold, where the boundary state has to be truncated
-        {"name": "truncated, d=17", "kind": "trunc", "d": 17, "chi": 32, "B": 2_048, "noise": "depol", "p": 0.12},
-        {"name": "truncated, d=25", "kind": "trunc", "d": 25, "chi": 64, "B": 515, "noise": "depol", "p": 0.12},
+        {"name": "truncated d=17", "kind": "trunc", "d": 17, "chi": 32, "B": 2_048, "noise": "depol", "p": 0.12},
+        {"name": "truncated d=25", "kind": "trunc", "d": 25, "chi": 64, "B": 515, "noise": "depol", "p": 0.12},
         # fitting a per-qubit noise model to labelled shots (forward and adjoint)
-        {"name": "labelled step, d=7", "kind": "train", "d": 7, "chi": 32, "B": 65_536, "labels": True},
+        {"name": "labelled step d=7", "kind": "train", "d": 7, "chi": 32, "B": 65_536, "labels": True},
         # the same from unlabelled shots, at the distance where the adjoint fills an SM
-        {"name": "unlabelled step, d=11", "kind": "train", "d": 11, "chi": 32, "B": 2_049, "labels": False},
+        {"name": "unlabelled step d=11", "kind": "train", "d": 11, "chi": 32, "B": 2_049, "labels": False},
         # a detector error model with X, Y and Z mechanisms on every qubit
-        {"name": "detector picture, d=9", "kind": "dem", "d": 9, "B": 65_536},
+        {"name": "detector picture d=9", "kind": "dem", "d": 9, "B": 65_536},
         # independent X/Z noise near threshold, in 32 bits
-        {"name": "independent XZ, d=17", "kind": "xz", "d": 17, "B": 8_191, "p": 0.10, "fp64": False, "bitflip": False},
+        {"name": "independent XZ d=17", "kind": "xz", "d": 17, "B": 8_191, "p": 0.10, "fp64": False, "bitflip": False},
         # the same noise at a lower rate on the largest patch, where 64 bits are asked for
-        {"name": "independent XZ, d=25", "kind": "xz", "d": 25, "B": 700, "p": 0.05, "fp64": True, "bitflip": False},
+        {"name": "independent XZ d=25", "kind": "xz", "d": 25, "B": 700, "p": 0.05, "fp64": True, "bitflip": False},
     ]
 
 
