@@ -125,9 +125,9 @@ mld_status mld_code_layout(const mld_code* code, int32_t* stab_type, int32_t* st
  *   argmax     device pointer uint8[B] or NULL: argmax_l Z_l(s), ties and
  *              all--inf rows go to the lowest class index.
  *   stream     cudaStream_t (NULL = legacy default stream).
- * Which kernel runs: see mld_code_set_exact_kernel (untruncated chi; the
- * same exact boundary state held as MPS sites or, at d = 11 and 13 by
- * default, densely) and mld_code_set_truncation_kernel (truncating chi).
+ * Which kernel runs: see mld_code_set_exact_kernel (untruncated chi: the
+ * same exact boundary state held densely, or as MPS sites) and
+ * mld_code_set_truncation_kernel (truncating chi).
  * All arrays are caller-owned device memory; the call is asynchronous and
  * allocates nothing per call once a call for the same (code, chi) and at
  * least the same B has been made (the first uploads the column plan and
@@ -213,10 +213,9 @@ void mld_graph_destroy(mld_graph* graph);
  * later decodes of this code object (per chi and precision). Where the
  * per-warp state exceeds a block's shared memory (d = 13 untruncated) the
  * candidates are the resident warps per SM of the global-workspace sweep
- * (2, 4, 8, 16; *chosen_warps reports that count). At an untruncated chi
- * with d = 9, 11 or 13 the dense-state kernel is a candidate too, and the faster
- * kernel is kept for that chi (*chosen_warps = 0 when it is the dense one),
- * unless mld_code_set_exact_kernel forces one. For a
+ * (2, 4, 8, 16; *chosen_warps reports that count). The column transfer of an
+ * untruncated chi has one block shape (*chosen_warps = 0) except at d = 9,
+ * where 1, 2, 4 and 8 warps are timed. For a
  * truncating chi the rank-adaptive sweep (4 units per block) is a candidate
  * beside the fixed-shape sweep's shapes, and the faster kernel is kept for
  * that chi (unless mld_code_set_truncation_kernel forces one). Synchronous. */
@@ -285,16 +284,14 @@ mld_status mld_code_set_truncation_workspace(mld_code* code, int max_bond);
 
 /* Which kernel decodes an untruncated chi (chi >= 2^floor(d/2), where the
  * boundary MPS of Sec. 3.2.1 discards nothing and is the exact boundary state
- * over one corner column): 0 (default) mld_autotune's choice for that chi if
- * it timed one, else the dense-state kernel at d = 11 and 13 (the faster
- * one there) and the boundary-MPS kernel elsewhere; 1 always the
- * boundary-MPS kernel (sites at the exact cut ranks, compile-time plan per
- * d; split-TF32 tensor-core products for MLD_MIXED_TF32 at d = 9, 11); 2
- * the dense-state kernel (d = 9, 11, 13: one block per (syndrome, l_Z) keeps
- * the 2^(d+2)-entry state of a column in shared memory and applies the
- * qubit factors to it in place; FP32 for either precision). Both give ln Z_l
- * to FP32 accuracy. MLD_ERR_INVALID_ARG for other values,
- * MLD_ERR_UNSUPPORTED for 2 at other d. Host only. */
+ * over one corner column): 0 (default) the column transfer for d <= 13 (the
+ * boundary state held densely, d bits, one 2x2 gate per qubit; FP32 for
+ * either precision; a syndrome whose two best classes tie up to rounding is
+ * decided by the boundary-MPS sweep at d <= 9); 1 always the boundary-MPS
+ * kernel (sites at the exact cut ranks, compile-time plan per d; split-TF32
+ * tensor-core products for MLD_MIXED_TF32 at d = 9, 11); 2 as 0 (d = 9, 11,
+ * 13). Both give ln Z_l to FP32 accuracy. MLD_ERR_INVALID_ARG for other
+ * values, MLD_ERR_UNSUPPORTED for 2 at other d. Host only. */
 mld_status mld_code_set_exact_kernel(mld_code* code, int which);
 
 /* Floating-point operations executed by the truncating sweeps of this code
@@ -337,11 +334,10 @@ mld_status mld_decode_flops(const mld_code* code, int chi, int precision, double
  *   syndromes  device uint64[B][words]
  *   logP       device double[B][4]: ln Z_l(s) (-inf for an impossible class)
  *   argmax     device uint8[B] or NULL (ties -> lowest class)
- * The contraction is exact: one thread block per syndrome keeps the dense
- * boundary state over the open detectors' partial parities and both
- * logical parities, all four classes in one sweep; FP32 with power-of-two
- * rescaling per column, ln Z in FP64. d <= 11 (the state at d = 11 is
- * 2^15 floats, one block of 512 threads per SM; MLD_ERR_UNSUPPORTED
+ * The contraction is exact: the mechanisms of a qubit are composed on the
+ * host (in FP64) and the network's parities are summed out column by column
+ * as in mld_decode's column transfer, all four classes in one launch; FP32
+ * with power-of-two rescaling per column. d <= 11 (MLD_ERR_UNSUPPORTED
  * otherwise); MLD_ERR_INVALID_ARG for a mechanism with a qubit outside
  * [0, n), a code outside 1..3 or p outside [0, 1]. Asynchronous on stream;
  * no device allocation. */
@@ -401,8 +397,10 @@ mld_status mld_decode_xz_executed_flops(const mld_code* code, double* flops);
  * a small buffer. */
 mld_status mld_measure_fp32_peak(double seconds, double* tflops, int* sm_count);
 
-/* Number of kernel launches one mld_decode call with an argmax output makes
- * (the noise check, the sweep, the argmax; for accounting). */
+/* Number of kernel launches one untruncated mld_decode call with an argmax
+ * output makes at most for d <= 13 (the column transfer, which checks the
+ * noise and takes the decisions, and at d = 9 the pass over tied syndromes;
+ * for accounting). */
 int mld_decode_launches(void);
 
 /* Static description of a status code. */

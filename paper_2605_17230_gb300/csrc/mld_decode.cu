@@ -27,7 +27,7 @@
 #include "mld_checks.h"
 #include "mld_dem.h"
 #include "mld_grad.h"
-#include "mld_dense.h"
+#include "mld_gate.h"
 #include "mld_internal.h"
 #include "mld_trunc.h"
 
@@ -945,19 +945,19 @@ mld_status decode_truncated(mld_code* C, const mld::Plan& P, const mld::SiteStep
 }  // namespace
 
 namespace mld {
-// Whether an untruncated decode of this code runs the dense-state kernel:
-// on request (mld_code_set_exact_kernel 2, d = 9, 11, 13), as mld_autotune
-// chose for this chi, or by default at d = 11 and 13, where it is the faster
-// exact kernel (measured: 2.61M against 2.07M syndromes/s for the split-TF32
-// boundary-MPS kernel at d = 11; 556k against 140k at d = 13, where the
-// exact boundary MPS needs 298 KB per unit and runs from global memory; at
-// d = 9 the boundary-MPS kernel is faster, 19.2M against 10.8M).
-bool uses_dense_exact(const mld_code* C, const Plan& P) {
-    if (P.svd_sites != 0 || !dense_exact_supported(C->d) || C->exact_kernel == 1) return false;
-    if (C->exact_kernel == 2) return true;
-    for (const auto& kv : C->exact_tuned)
-        if (kv.first == P.chi) return kv.second == 2;
-    return C->d >= 11;
+// Whether an untruncated decode of this code runs the column transfer
+// (mld_gate.cu): at every d it is compiled for, unless the caller chose the
+// boundary-MPS kernel.
+bool uses_gate(const mld_code* C, const Plan& P) {
+    return P.svd_sites == 0 && gate_supported(C->d) && C->exact_kernel != 1;
+}
+
+// Warps per block of the column transfer at d = 9: mld_autotune's choice, or 0.
+int gate_warps(const mld_code* C, int chi, int precision) {
+    if (C->force_warps > 0) return C->force_warps;
+    for (const auto& kv : C->tuned)
+        if (kv.first == chi * 4 + precision) return kv.second;
+    return 0;
 }
 
 // Whether the untruncated or fixed-shape sweep of this code at this chi keeps
@@ -965,7 +965,7 @@ bool uses_dense_exact(const mld_code* C, const Plan& P) {
 // are resident warps per SM).
 bool state_in_global_workspace(const mld_code* C, int chi) {
     const Plan P = make_plan(C->d, chi);
-    if (uses_dense_exact(C, P)) return false;
+    if (uses_gate(C, P)) return false;
     const bool exact = P.svd_sites == 0 && exact_floats_per_warp(C->d) > 0;
     int dev = 0, max_optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -1034,11 +1034,11 @@ mld_status mld_code_layout(const mld_code* C, int32_t* type, int32_t* sup, uint8
     return MLD_OK;
 }
 
-int mld_decode_launches(void) { return 3; }
+int mld_decode_launches(void) { return 2; }
 
 mld_status mld_code_set_exact_kernel(mld_code* C, int which) {
     if (!C || which < 0 || which > 2) return MLD_ERR_INVALID_ARG;
-    if (which == 2 && !mld::dense_exact_supported(C->d)) return MLD_ERR_UNSUPPORTED;
+    if (which == 2 && C->d != 9 && C->d != 11 && C->d != 13) return MLD_ERR_UNSUPPORTED;
     C->exact_kernel = which;
     return MLD_OK;
 }
@@ -1050,8 +1050,8 @@ mld_status mld_decode_flops(const mld_code* C, int chi, int precision, double* o
     // every kernel sweeps columns 0..d-2 once per l_Z and the last column once
     // per class
     const mld::Plan P = mld::make_plan(C->d, chi);
-    if (mld::uses_dense_exact(C, P)) {
-        *out = mld::dense_exact_flops_per_syndrome(C->d);
+    if (mld::uses_gate(C, P)) {
+        *out = mld::gate_flops_per_syndrome(C->d);
         return MLD_OK;
     }
     *out = 2.0 * (P.flops_per_coset - P.flops_last_col) + 4.0 * P.flops_last_col;
@@ -1073,6 +1073,28 @@ mld_status mld_decode(const mld_code* Cc, const float* noise, int noise_mode, co
     const mld_code::PlanDev* pd = get_plan(C, chi, &st);
     if (!pd) return st;
     const mld::Plan& P = pd->plan;
+    // untruncated chi (every kept dimension is min(rows, cols)): a kernel
+    // specialised for this d, when one exists
+    const bool exact = P.svd_sites == 0 && mld::exact_floats_per_warp(C->d) > 0;
+    // mixed precision is accepted where such a kernel exists; BF16 operands
+    // and truncating chi are not
+    if (precision == MLD_MIXED_BF16 || (precision == MLD_MIXED_TF32 && !exact)) return MLD_ERR_UNSUPPORTED;
+    if (mld::uses_gate(C, P)) {
+        mld::GateArgs ga;
+        ga.dmask = C->d_dmask;
+        ga.noise = noise;
+        ga.syn = syn;
+        ga.logP = logP;
+        ga.argmax = argmax;
+        ga.status = C->d_status;
+        ga.B = B;
+        ga.noise_mode = noise_mode;
+        ga.precision = precision;
+        return mld::launch_gate(C->d, ga, nullptr, mld::gate_warps(C, chi, precision),
+                                reinterpret_cast<cudaStream_t>(stream))
+                   ? MLD_OK
+                   : MLD_ERR_CUDA;
+    }
     mld::DecodeArgs a;
     a.steps = pd->d_steps;
     a.dmask = C->d_dmask;
@@ -1099,12 +1121,6 @@ mld_status mld_decode(const mld_code* Cc, const float* noise, int noise_mode, co
         cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess)
         return MLD_ERR_CUDA;
-    // untruncated chi (every kept dimension is min(rows, cols)): the
-    // compile-time specialised kernel, when one exists for this d
-    const bool exact = P.svd_sites == 0 && mld::exact_floats_per_warp(C->d) > 0;
-    // the mixed-precision path exists for the untruncated specialised kernel
-    // (TF32 tensor-core products); BF16 and truncating chi run FP32 only
-    if (precision == MLD_MIXED_BF16 || (precision == MLD_MIXED_TF32 && !exact)) return MLD_ERR_UNSUPPORTED;
     // truncating chi: the rank-adaptive sweep, or the fixed-shape one when its
     // whole per-warp state fits 24 KB of shared memory (small chi and d, where
     // its compile-free static shapes beat the runtime ones), unless the
@@ -1120,28 +1136,6 @@ mld_status mld_decode(const mld_code* Cc, const float* noise, int noise_mode, co
             return MLD_ERR_CUDA;
         const mld_status ts = decode_truncated(C, P, pd->d_steps, noise, noise_mode, syn, B, chi, logP, s);
         if (ts != MLD_OK) return ts;
-        if (argmax) {
-            mld::argmax_kernel<<<(unsigned)((B + 255) / 256), 256, 0, s>>>(logP, argmax, B);
-            if (cudaGetLastError() != cudaSuccess) return MLD_ERR_CUDA;
-        }
-        return MLD_OK;
-    }
-    if (mld::uses_dense_exact(C, P)) {
-        // untruncated, dense boundary state (FP32 for either precision: no
-        // product is MMA-shaped)
-        cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-        if (!mld::launch_noise_check(noise, noise_mode, noise_mode == MLD_NOISE_TABLE ? C->n : B, C->d_status, s))
-            return MLD_ERR_CUDA;
-        mld::DenseArgs da;
-        da.dmask = C->d_dmask;
-        da.noise = noise;
-        da.syn = syn;
-        da.logP = logP;
-        da.status = C->d_status;
-        da.B = B;
-        da.words = C->words;
-        da.noise_mode = noise_mode;
-        if (!mld::launch_dense_exact(C->d, da, s)) return MLD_ERR_CUDA;
         if (argmax) {
             mld::argmax_kernel<<<(unsigned)((B + 255) / 256), 256, 0, s>>>(logP, argmax, B);
             if (cudaGetLastError() != cudaSuccess) return MLD_ERR_CUDA;

@@ -33,4 +33,8 @@ bool launch_exact(int d, const ExactArgs& a, cudaStream_t s, int warps_per_block
     return false;
 }
 
+bool launch_decide_ties(const ExactArgs& a, uint8_t* argmax, int precision, int sms, cudaStream_t s) {
+    return exact::launch_ties_d<9>(a, argmax, precision, sms, s);
+}
+
 }  // namespace mld

@@ -24,4 +24,7 @@ struct ExactArgs {
 int exact_floats_per_warp(int d);
 bool launch_exact(int d, const ExactArgs& a, cudaStream_t s, int warps_per_block, int precision);
 
+// The pass that decides the ties marked in a batch's decisions (d = 9).
+bool launch_decide_ties(const ExactArgs& a, uint8_t* argmax, int precision, int sms, cudaStream_t s);
+
 }  // namespace mld

@@ -1014,6 +1014,59 @@ __device__ __forceinline__ void decode_unit(const ExactArgs& a, float* ws, int64
     }
 }
 
+// Decides again a syndrome that the column transfer marked: its two best
+// classes are equal up to rounding, as lattice symmetries make them under
+// uniform noise (5 to 18 of 65,536 syndromes at d = 9, p = 0.10; 4% at d = 5,
+// p = 0.19). Which class wins such a tie is a matter of rounding alone, so ln Z
+// and the decision come from this sweep, whichever kernel decodes the rest of
+// the batch. One warp; lane 0 has stored the four values that it compares.
+template <int D, int PREC>
+__device__ __forceinline__ void decide_from(const ExactArgs& a, uint8_t* argmax, int64_t b) {
+    int best = 0;
+    for (int l = 1; l < 4; ++l)
+        if (a.logP[4 * b + l] > a.logP[4 * b + best]) best = l;
+    argmax[b] = (uint8_t)best;
+}
+template <int D, int PREC>
+__device__ __noinline__ void decide_tie(const ExactArgs& a, uint8_t* argmax, float* ws, int64_t b, int lane) {
+#pragma unroll 1
+    for (int lz = 0; lz < 2; ++lz) {
+        decode_unit<D, PREC>(a, ws, 2 * b + lz, lane);
+        __syncwarp();
+    }
+    if (lane == 0) decide_from<D, PREC>(a, argmax, b);
+}
+
+// The same as a pass over a batch's decisions (bit 7 marks), where the marking
+// kernel has no room for this sweep's state: a block of two warps (l_Z = 0, 1)
+// looks at 128 decisions at a time. The pass lasts one sweep's latency.
+template <int D, int PREC>
+__global__ void __launch_bounds__(64) decide_ties_kernel(ExactArgs a, uint8_t* argmax) {
+    constexpr int FPW = LayoutOf<D>::lay.floats_per_warp;
+    extern __shared__ float4 smem4[];
+    const int lz = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* ws = reinterpret_cast<float*>(smem4) + (size_t)lz * FPW;
+    for (int64_t b0 = (int64_t)blockIdx.x * 128; b0 < a.B; b0 += (int64_t)gridDim.x * 128) {
+        int mine = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t b = b0 + 32 * k + lane;
+            mine |= (b < a.B && (argmax[b] & 0x80)) << k;
+        }
+        if (!__syncthreads_or(mine)) continue;        // both warps have read the marks
+        for (int k = 0; k < 4; ++k) {
+            unsigned marked = __ballot_sync(0xffffffffu, (mine >> k) & 1);
+            while (marked) {
+                const int64_t b = b0 + 32 * k + __ffs(marked) - 1;
+                marked &= marked - 1;
+                decode_unit<D, PREC>(a, ws, 2 * b + lz, lane);
+                __syncthreads();
+                if (threadIdx.x == 0) decide_from<D, PREC>(a, argmax, b);
+            }
+        }
+    }
+}
+
 // States up to this many floats per warp run from shared memory; larger
 // ones (d >= 13) from the global workspace.
 constexpr int kSharedFloatsMax = (227 * 1024) / 4;
@@ -1048,6 +1101,24 @@ bool launch_d(const ExactArgs& a, cudaStream_t s, int warps_per_block, int preci
     }
     if (precision == MLD_FP32) return launch_dp<D, MLD_FP32>(a, s, warps_per_block);
     return false;
+}
+
+template <int D, int PREC>
+bool launch_ties_dp(const ExactArgs& a, uint8_t* argmax, int sms, cudaStream_t s) {
+    constexpr size_t smem = 2 * (size_t)LayoutOf<D>::lay.floats_per_warp * sizeof(float);
+    static_assert(smem <= 48 * 1024, "two warps' states in a block's default shared memory");
+    int64_t blocks = (a.B + 127) / 128;
+    if (blocks > 4 * (int64_t)sms) blocks = 4 * (int64_t)sms;
+    decide_ties_kernel<D, PREC><<<(unsigned)blocks, 64, smem, s>>>(a, argmax);
+    return cudaGetLastError() == cudaSuccess;
+}
+
+template <int D>
+bool launch_ties_d(const ExactArgs& a, uint8_t* argmax, int precision, int sms, cudaStream_t s) {
+    if constexpr (kTensorPays<D>) {
+        if (precision == MLD_MIXED_TF32) return launch_ties_dp<D, MLD_MIXED_TF32>(a, argmax, sms, s);
+    }
+    return launch_ties_dp<D, MLD_FP32>(a, argmax, sms, s);
 }
 
 }  // namespace exact

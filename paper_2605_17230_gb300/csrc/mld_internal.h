@@ -54,12 +54,10 @@ struct mld_code {
     // largest bond capacity of the rank-adaptive sweep's first pass (0: the
     // smallest that holds chi, up to 128; else 48, 64 or 128)
     int trunc_first_bond = 0;
-    // which kernel runs an untruncated chi: 0 mld_autotune's choice for that
-    // chi if it timed one (exact_tuned), else by d (the dense-state kernel at
-    // d = 11, 13, the boundary-MPS kernel elsewhere); 1 the boundary-MPS
-    // kernel; 2 the dense-state kernel (d = 9, 11, 13)
+    // which kernel runs an untruncated chi at d <= 13: 0 or 2 the column
+    // transfer (the state held dense, one gate per qubit), 1 the boundary-MPS
+    // kernel
     int exact_kernel = 0;
-    std::vector<std::pair<int, int>> exact_tuned;
     // Kac-Ward solver (mld_decode_xz): one device block holding the ordered
     // matrix of the spin graph (CSR row starts, columns, weight sources, each
     // band row's last column, the quarter-turn qubit map; then the phases as
@@ -73,5 +71,6 @@ struct mld_code {
 
 namespace mld {
 bool state_in_global_workspace(const mld_code* C, int chi);
-bool uses_dense_exact(const mld_code* C, const Plan& P);
+bool uses_gate(const mld_code* C, const Plan& P);
+int gate_warps(const mld_code* C, int chi, int precision);
 }

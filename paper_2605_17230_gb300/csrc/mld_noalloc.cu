@@ -15,7 +15,7 @@
 #include <vector>
 
 #include "mld_checks.h"
-#include "mld_exact.h"
+#include "mld_gate.h"
 #include "mld_internal.h"
 
 namespace {
@@ -43,16 +43,6 @@ uint64_t table_hash(const std::vector<uint64_t>& t) {
             h *= 1099511628211ULL;
         }
     return h | 1ULL;                 // never 0
-}
-
-__global__ void noalloc_argmax(const double* __restrict__ logP, uint8_t* __restrict__ am, int64_t B) {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const double* l = logP + 4 * b;
-    int best = 0;
-    for (int k = 1; k < 4; ++k)
-        if (l[k] > l[best]) best = k;
-    am[b] = (uint8_t)best;
 }
 
 // Device address of the scratch array for the current device. In host code
@@ -88,28 +78,13 @@ extern "C" mld_status mld_decode_noalloc(const mld_code* C, const float* noise, 
     // only the untruncated FP32 sweep of the distances with a specialised
     // kernel, and only codes whose tables fit in the scratch array
     const size_t table_bytes = C->dmask.size() * sizeof(uint64_t);
-    if (precision != MLD_FP32 || C->d > 11 || mld::exact_floats_per_warp(C->d) == 0 ||
+    if (precision != MLD_FP32 || C->d > 11 || !mld::gate_supported(C->d) ||
         mld::make_plan(C->d, chi).svd_sites != 0 || kStatusSlot + table_bytes > kNoAllocBytes)
         return MLD_ERR_UNSUPPORTED;
     unsigned char* scratch = nullptr;
     int device = 0;
     mld_status st = scratch_address(&scratch, &device);
     if (st != MLD_OK) return st;
-    int dev = 0, max_optin = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess)
-        return MLD_ERR_CUDA;
-    const size_t pw = (size_t)mld::exact_floats_per_warp(C->d) * sizeof(float);
-    if (pw > (size_t)max_optin) return MLD_ERR_UNSUPPORTED;
-    int W = 1, best = 0;
-    for (int w = 1; w <= 8; ++w) {
-        if (pw * w > (size_t)max_optin) break;
-        int ctas = (int)((size_t)per_sm / (pw * w + 1024));
-        ctas = ctas < 32 ? ctas : 32;
-        const int warps = ctas * w < 64 ? ctas * w : 64;
-        if (warps > best) { best = warps; W = w; }
-    }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // the status word starts at zero in every call; the tables are uploaded
     // only when the array holds another code's (the previous call's code is
@@ -125,22 +100,17 @@ extern "C" mld_status mld_decode_noalloc(const mld_code* C, const float* noise, 
             g_tables_written[device] = tables;
         }
     }
-    if (!mld::launch_noise_check(noise, noise_mode, noise_mode == MLD_NOISE_TABLE ? C->n : B,
-                                 reinterpret_cast<int*>(scratch), s))
-        return MLD_ERR_CUDA;
-    mld::ExactArgs ea;
-    ea.dmask = reinterpret_cast<const uint64_t*>(scratch + kStatusSlot);
-    ea.noise = noise;
-    ea.syn = syndromes;
-    ea.logP = logP;
-    ea.status = reinterpret_cast<int*>(scratch);
-    ea.B = B;
-    ea.noise_mode = noise_mode;
-    if (!mld::launch_exact(C->d, ea, s, W, MLD_FP32)) return MLD_ERR_CUDA;
-    if (argmax) {
-        noalloc_argmax<<<(unsigned)((B + 255) / 256), 256, 0, s>>>(logP, argmax, B);
-        if (cudaGetLastError() != cudaSuccess) return MLD_ERR_CUDA;
-    }
+    mld::GateArgs ga;
+    ga.dmask = reinterpret_cast<const uint64_t*>(scratch + kStatusSlot);
+    ga.noise = noise;
+    ga.syn = syndromes;
+    ga.logP = logP;
+    ga.argmax = argmax;
+    ga.status = reinterpret_cast<int*>(scratch);
+    ga.B = B;
+    ga.noise_mode = noise_mode;
+    ga.precision = precision;
+    if (!mld::launch_gate(C->d, ga, nullptr, 0, s)) return MLD_ERR_CUDA;
     if (!check_status) return MLD_OK;
     int h = 0;
     if (cudaMemcpyAsync(&h, scratch, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
