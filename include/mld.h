@@ -345,8 +345,8 @@ mld_status mld_decode_dem(const mld_code* code, const int32_t* mech_qubit, const
                           const double* mech_p, int32_t n_mech, const uint64_t* syndromes, int64_t B,
                           double* logP, uint8_t* argmax, void* stream);
 
-/* MLD under independent X/Z noise by Kac-Ward determinants (Sec. 3.1.3:
- * the planar random-bond Ising model of each part, Z proportional to
+/* MLD under independent X/Z noise (Sec. 3.1.3: the planar random-bond Ising
+ * model of each part; with Kac-Ward determinants, Z is proportional to
  * sqrt(det(I - Lambda)) per logical sector). Qubit q flips its X part with
  * probability px[q] and its Z part with probability pz[q], independently:
  * Pr(E) = prod_q px^x (1-px)^(1-x) pz^z (1-pz)^(1-z), so the class
@@ -358,11 +358,14 @@ mld_status mld_decode_dem(const mld_code* code, const int32_t* mech_qubit, const
  *              errors): ln Z is -inf for l_Z = 1, and for every class of a
  *              syndrome whose X-type part is nonzero
  *   syndromes  device uint64[B][words]
- *   precision  MLD_FP32 or MLD_FP64 (complex arithmetic of that type)
+ *   precision  MLD_FP32: Kac-Ward determinants in complex FP32; MLD_FP64:
+ *              the parts' column transfer at FP64 accuracy (accurate at
+ *              every rate, and the faster one: d = 25 233 k syndromes/s
+ *              against 69 k)
  *   logP       device double[B][4]: ln Z_l(s)
  *   argmax     device uint8[B] or NULL (ties -> lowest class)
- * Exact in exact arithmetic at any odd d >= 3 up to 25. Each part is one
- * banded elimination with partial pivoting (order 2|E| = 2d^2 + O(d),
+ * Exact in exact arithmetic at any odd d >= 3 up to 25. MLD_FP32: each part is
+ * one banded elimination with partial pivoting (order 2|E| = 2d^2 + O(d),
  * bandwidth 3d), one warp per syndrome up to d = 13 and one block of four
  * warps per syndrome above, the two sectors sharing all but a final 4 x 4
  * determinant. The determinant is a sum of signed terms, so accuracy
@@ -372,22 +375,25 @@ mld_status mld_decode_dem(const mld_code* code, const int32_t* mech_qubit, const
  * MLD_FP64 (4,096 syndromes per point): MLD_FP32 keeps the leading ln Z
  * within 1.1e-3 at p = 0.10 up to d = 25, but on rare syndromes reaches
  * 0.097 (p = 0.05) and 0.29 (p = 0.02) at d = 25; one decision in 4,096
- * differed at d = 17, p = 0.02. Use MLD_FP64 for ln Z at low rates. A probability
- * outside (0, 1) sets MLD_ERR_INVALID_ARG in the status word
- * (mld_decode_status); a vanishing pivot sets MLD_ERR_NUMERIC and gives -inf.
- * The first call for a code builds the graph and copies it to the device
- * (synchronous, a few hundred KB); later calls are asynchronous on stream
- * with no allocation. MLD_ERR_UNSUPPORTED if a syndrome's window exceeds
- * the device's shared memory per block (it fits up to d = 25 in FP64 on
- * GB300: 200 KB). */
+ * differed at d = 17, p = 0.02. MLD_FP64: each part's partition function is
+ * swept column by column over (d-1)/2 bits, every term positive, in FP64 up
+ * to d = 13 and in pairs of FP32 numbers above (relative error of Z some
+ * 1e-13); use it for ln Z at low rates and for the less likely classes. A
+ * probability outside (0, 1) sets MLD_ERR_INVALID_ARG in the status word
+ * (mld_decode_status); a vanishing pivot or sum sets MLD_ERR_NUMERIC and
+ * gives -inf. The first call of a precision for a code builds its tables and
+ * copies them to the device (synchronous, a few hundred KB); later calls are
+ * asynchronous on stream with no allocation. MLD_ERR_UNSUPPORTED if a
+ * syndrome's state exceeds the device's shared memory per block (it fits up
+ * to d = 25 on GB300). */
 mld_status mld_decode_xz(const mld_code* code, const float* px, const float* pz, const uint64_t* syndromes,
                          int64_t B, int precision, double* logP, uint8_t* argmax, void* stream);
 
 /* Floating-point operations executed by mld_decode_xz on this code since the
  * last call (per elimination step: a complex multiplier, 6 flops, and a
  * complex multiply-subtract, 8 flops, per updated column of every row with a
- * nonzero multiplier, counted on the device from the step's actual extent),
- * then reset to zero. The caller synchronises the decode streams first. */
+ * nonzero multiplier, counted on the device from the step's actual extent;
+ * MLD_FP64: three per state entry and gate), then reset to zero. The caller synchronises the decode streams first. */
 mld_status mld_decode_xz_executed_flops(const mld_code* code, double* flops);
 
 /* Measurement helper (not part of the method): times a kernel of independent

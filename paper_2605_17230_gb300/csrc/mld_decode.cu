@@ -1008,6 +1008,7 @@ void mld_code_destroy(mld_code* C) {
         cudaFree(C->d_tctl);
         cudaFree(C->d_ovf);
         cudaFree(C->d_kw);
+        cudaFree(C->d_xz);
     }
     delete C;
 }

@@ -58,15 +58,20 @@ struct mld_code {
     // transfer (the state held dense, one gate per qubit), 1 the boundary-MPS
     // kernel
     int exact_kernel = 0;
-    // Kac-Ward solver (mld_decode_xz): one device block holding the ordered
-    // matrix of the spin graph (CSR row starts, columns, weight sources, each
-    // band row's last column, the quarter-turn qubit map; then the phases as
-    // double pairs at kw_ph_off; an executed-flop counter at kw_cnt_off),
+    // Kac-Ward solver (mld_decode_xz, MLD_FP32): one device block holding the
+    // ordered matrix of the spin graph (CSR row starts, columns, weight sources,
+    // each band row's last column, the quarter-turn qubit map; then the phases
+    // as double pairs at kw_ph_off; an executed-flop counter at kw_cnt_off),
     // built on first use, and its sizes
     void* d_kw = nullptr;
     int kw_N = 0, kw_Nb = 0, kw_bl = 0, kw_bu = 0, kw_nplaq = 0, kw_nnz = 0;
     size_t kw_ph_off = 0;
     size_t kw_cnt_off = 0;               // executed-flop counter (double) in the same block
+    // transfer under independent X/Z noise (mld_decode_xz, MLD_FP64), made on first use:
+    // representative masks in processing order (xz_masks words), the X-type
+    // checks (words), an executed-flop counter (double)
+    uint64_t* d_xz = nullptr;
+    size_t xz_masks = 0;
 };
 
 namespace mld {

@@ -28,7 +28,8 @@
 // values) are carried beside the window, so both sectors share every step
 // but the last: a 4 x 4 determinant per sector (the two remaining band rows,
 // the two border rows). ln|det| accumulates the pivots' squared moduli as a
-// mantissa and a power-of-two exponent. Complex FP32 or FP64.
+// mantissa and a power-of-two exponent. Complex FP32; FP64 requests run the
+// column transfer (mld_xz.cu), whose terms are all positive.
 //
 // Floating point: ES sums signed terms, so the elimination loses accuracy
 // with the conditioning of I - Lambda: a class far less likely than the
@@ -37,8 +38,7 @@
 // even the leading class can: measured against FP64 over 4,096 syndromes,
 // complex FP32 keeps the leading ln Z within 1.1e-3 at p = 0.10 up to d = 25,
 // but reaches 0.097 (p = 0.05) and 0.29 (p = 0.02) at d = 25 on rare
-// syndromes, and one decision of 4,096 differed at d = 17, p = 0.02. FP64 is
-// the accurate mode.
+// syndromes, and one decision of 4,096 differed at d = 17, p = 0.02.
 #include <math.h>
 #include <stdint.h>
 
@@ -50,6 +50,7 @@
 #include "mld_dem.h"
 #include "mld_internal.h"
 #include "mld_kw.h"
+#include "mld_xz.h"
 
 namespace mld {
 
@@ -211,10 +212,6 @@ struct Cplx;
 template <>
 struct Cplx<float> {
     using type = float2;
-};
-template <>
-struct Cplx<double> {
-    using type = double2;
 };
 
 constexpr int kKwMaxColsPerLane = 5;   // (bl + bu) / 32 rounded up; 5 covers d <= 25
@@ -1206,6 +1203,8 @@ extern "C" mld_status mld_decode_xz(const mld_code* Cc, const float* px, const f
     if (!px || !syndromes || !logP) return MLD_ERR_INVALID_ARG;
     mld_status st = ensure_code_device(C);
     if (st != MLD_OK) return st;
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    if (precision == MLD_FP64) return decode_xz_fp64(C, px, pz, syndromes, B, logP, argmax, s);
     st = ensure_kw(C);
     if (st != MLD_OK) return st;
     KwArgs a;
@@ -1235,17 +1234,18 @@ extern "C" mld_status mld_decode_xz(const mld_code* Cc, const float* px, const f
     a.argmax = argmax;
     a.status = C->d_status;
     a.flops = reinterpret_cast<double*>(reinterpret_cast<char*>(C->d_kw) + C->kw_cnt_off);
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    return precision == MLD_FP64 ? launch_kw<double>(a, s) : launch_kw<float>(a, s);
+    return launch_kw<float>(a, s);
 }
 
 extern "C" mld_status mld_decode_xz_executed_flops(const mld_code* Cc, double* out) {
     mld_code* C = const_cast<mld_code*>(Cc);
     if (!C || !out) return MLD_ERR_INVALID_ARG;
-    *out = 0.0;
-    if (!C->d_kw) return MLD_OK;
+    const mld_status st = mld::xz_fp64_flops(C, out);
+    if (st != MLD_OK || !C->d_kw) return st;
     char* cnt = static_cast<char*>(C->d_kw) + C->kw_cnt_off;
-    if (cudaMemcpy(out, cnt, sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) return MLD_ERR_CUDA;
+    double kw = 0.0;
+    if (cudaMemcpy(&kw, cnt, sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) return MLD_ERR_CUDA;
+    *out += kw;
     if (cudaMemset(cnt, 0, sizeof(double)) != cudaSuccess) return MLD_ERR_CUDA;
     return MLD_OK;
 }
