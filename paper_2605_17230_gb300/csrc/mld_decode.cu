@@ -1279,39 +1279,42 @@ mld_status mld_decode_grad(const mld_code* Cc, const float* noise, const uint64_
     const mld::Plan& P = pd->plan;
     if (P.svd_sites != 0) return MLD_ERR_UNSUPPORTED;       // exact environments need untruncated chi
     const int d = C->d, n = C->n;
-    if (!mld::launch_noise_check(noise, MLD_NOISE_TABLE, n, C->d_status, reinterpret_cast<cudaStream_t>(stream)))
-        return MLD_ERR_CUDA;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return MLD_ERR_CUDA;
-    if (!mld::grad_dense_supported(d)) return MLD_ERR_UNSUPPORTED;
-    {
-        // dense states (on chip, or in the block's global slice at d = 13): one
-        // block per (syndrome, class) unit
-        const int64_t blocks = mld::grad_dense_blocks(d, sms, B);
-        if (blocks < 1) return MLD_ERR_CUDA;
-        const size_t bytes = (size_t)blocks * mld::grad_dense_workspace_floats(d) * sizeof(float);
-        if (bytes > C->gradws_bytes) {
-            cudaFree(C->d_gradws);
-            C->d_gradws = nullptr;
-            C->gradws_bytes = 0;
-            if (cudaMalloc(&C->d_gradws, bytes) != cudaSuccess) return MLD_ERR_NOMEM;
-            C->gradws_bytes = bytes;
-        }
-        mld::GradDenseArgs ga;
-        ga.dmask = C->d_dmask;
-        ga.noise = noise;
-        ga.syn = syn;
-        ga.dlogP = dlogP;
-        ga.logP = logP;
-        ga.dnoise = dnoise;
-        ga.lws = C->d_gradws;
-        ga.B = B;
-        ga.words = C->words;
-        return mld::launch_grad_dense(d, ga, blocks, reinterpret_cast<cudaStream_t>(stream)) ? MLD_OK
-                                                                                              : MLD_ERR_CUDA;
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    const bool gate = d <= 11;           // states in registers; d = 13: in a block's global slice
+    int64_t blocks = 0;
+    if (gate) {
+        blocks = mld::grad_gate_blocks(d, B);
+    } else {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return MLD_ERR_CUDA;
+        blocks = mld::grad_dense_blocks(d, sms, B);
+        if (!mld::launch_noise_check(noise, MLD_NOISE_TABLE, n, C->d_status, s)) return MLD_ERR_CUDA;
     }
+    if (blocks < 1) return MLD_ERR_CUDA;
+    const size_t bytes = (size_t)blocks * sizeof(float) *
+                         (gate ? mld::grad_gate_workspace_floats(d) : mld::grad_dense_workspace_floats(d));
+    if (bytes > C->gradws_bytes) {
+        cudaFree(C->d_gradws);
+        C->d_gradws = nullptr;
+        C->gradws_bytes = 0;
+        if (cudaMalloc(&C->d_gradws, bytes) != cudaSuccess) return MLD_ERR_NOMEM;
+        C->gradws_bytes = bytes;
+    }
+    mld::GradDenseArgs ga;
+    ga.dmask = C->d_dmask;
+    ga.noise = noise;
+    ga.syn = syn;
+    ga.dlogP = dlogP;
+    ga.logP = logP;
+    ga.dnoise = dnoise;
+    ga.lws = C->d_gradws;
+    ga.status = C->d_status;
+    ga.B = B;
+    ga.words = C->words;
+    const bool ok = gate ? mld::launch_grad_gate(d, ga, blocks, s) : mld::launch_grad_dense(d, ga, blocks, s);
+    return ok ? MLD_OK : MLD_ERR_CUDA;
 }
 
 mld_status mld_code_set_svd_cutoff(mld_code* C, double rel) {

@@ -185,7 +185,7 @@ __device__ __forceinline__ void thread_body(const GateArgs& a, const float4* tab
                 const auto w = [&](int T) { return weight(c, D - 2 - T, word); };
                 if constexpr (S::NB >= 2) gates_down<S::NB, S::NB - 2>(P, w);
                 gate_pair<S::NB>(P, weight(c, D - 1, word));
-                sc = rescale(__float_as_uint(max_of(P)), e2);
+                sc = rescale<>(__float_as_uint(max_of(P)), e2);
             }
 #pragma unroll
             for (int k = 0; k + 1 < S::PAIRS; ++k) W[k] = W[k + 1];
@@ -196,7 +196,7 @@ __device__ __forceinline__ void thread_body(const GateArgs& a, const float4* tab
                 gate_pair<S::NB>(P, v);
                 const auto w = [&](int T) { return weight(c, T + 1, W[0]); };
                 gates_up<S::NB, 0>(P, w);
-                sc = rescale(__float_as_uint(max_of(P)), e2);
+                sc = rescale<>(__float_as_uint(max_of(P)), e2);
             }
         }
         // last column, both l_X at once: X on the column flips row 0's new bit,
@@ -449,7 +449,7 @@ __device__ __forceinline__ void lane_body(const GateArgs& a, const float4* table
             if constexpr (S::LANES == 64)
                 mx = max(__float_as_uint(pair_x[lz * 8]), __float_as_uint(pair_x[lz * 8 + 1]));
             unit_sync<D>(lz);
-            const float sc = rescale(mx, e2);
+            const float sc = rescale<>(mx, e2);
             float4 v = weight(c, M + 1, word, 0);
             v = make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
             gate_bit<M, 0>(P, v);

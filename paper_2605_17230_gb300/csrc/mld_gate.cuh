@@ -203,8 +203,9 @@ __device__ __forceinline__ double ln_scaled(float z, int e) {
 // d = 11 these lie up to e^-110 below the largest). Returns the factor and
 // takes its logarithm off the exponent.
 constexpr int kTop = 100;
+template <int TOP = kTop>
 __device__ __forceinline__ float rescale(uint32_t mbits, int& e2) {
-    int up = mbits ? kTop + 127 - (int)(mbits >> 23) : 0;
+    int up = mbits ? TOP + 127 - (int)(mbits >> 23) : 0;
     up = up > 127 ? 127 : up;
     e2 -= up;
     return __uint_as_float((uint32_t)(127 + up) << 23);

@@ -595,15 +595,8 @@ bool launch_d(const GradDenseArgs& a, int64_t blocks, cudaStream_t s) {
 
 }  // namespace
 
-bool grad_dense_supported(int d) { return d == 3 || d == 5 || d == 7 || d == 9 || d == 11 || d == 13; }
-
 int64_t grad_dense_blocks(int d, int sms, int64_t B) {
     switch (d) {
-        case 3: return blocks_d<3>(sms, B);
-        case 5: return blocks_d<5>(sms, B);
-        case 7: return blocks_d<7>(sms, B);
-        case 9: return blocks_d<9>(sms, B);
-        case 11: return blocks_d<11>(sms, B);
         case 13: return blocks_d<13>(sms, B);
     }
     return 0;
@@ -611,11 +604,6 @@ int64_t grad_dense_blocks(int d, int sms, int64_t B) {
 
 int64_t grad_dense_workspace_floats(int d) {
     switch (d) {
-        case 3: return GradShape<3>::slice;
-        case 5: return GradShape<5>::slice;
-        case 7: return GradShape<7>::slice;
-        case 9: return GradShape<9>::slice;
-        case 11: return GradShape<11>::slice;
         case 13: return GradShape<13>::slice;
     }
     return 0;
@@ -623,11 +611,6 @@ int64_t grad_dense_workspace_floats(int d) {
 
 bool launch_grad_dense(int d, const GradDenseArgs& a, int64_t blocks, cudaStream_t s) {
     switch (d) {
-        case 3: return launch_d<3>(a, blocks, s);
-        case 5: return launch_d<5>(a, blocks, s);
-        case 7: return launch_d<7>(a, blocks, s);
-        case 9: return launch_d<9>(a, blocks, s);
-        case 11: return launch_d<11>(a, blocks, s);
         case 13: return launch_d<13>(a, blocks, s);
     }
     return false;

@@ -215,7 +215,7 @@ struct Range<Twin> {
     static constexpr int top = gate::kTop;
     static __device__ __forceinline__ Twin start() { return Twin{gate::top_scale(), 0.f}; }
     static __device__ __forceinline__ uint32_t bits(Twin v) { return __float_as_uint(v.hi); }
-    static __device__ __forceinline__ float rescale(uint32_t m, int& e2) { return gate::rescale(m, e2); }
+    static __device__ __forceinline__ float rescale(uint32_t m, int& e2) { return gate::rescale<>(m, e2); }
 };
 template <typename T, int N>
 __device__ __forceinline__ uint32_t max_bits(const T (&v)[N]) {
