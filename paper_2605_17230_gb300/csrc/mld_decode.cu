@@ -819,7 +819,6 @@ mld_status grow(T** buf, size_t* have, size_t bytes) {
 // pass 1, [20] of pass 2, [24] executed flops (f64, accumulated), [32] bond
 // histogram (65 x u64, accumulated).
 constexpr size_t kTctlBytes = 1024;
-constexpr int kTruncArena = 3072;        // on-chip work arena per unit (floats)
 
 mld_status decode_truncated(mld_code* C, const mld::Plan& P, const mld::SiteStep* d_steps, const float* noise,
                             int noise_mode, const uint64_t* syn, int64_t B, int chi, double* logP,
@@ -829,7 +828,8 @@ mld_status decode_truncated(mld_code* C, const mld::Plan& P, const mld::SiteStep
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return MLD_ERR_CUDA;
     const int64_t units = 2 * B;
-    const int bps = mld::trunc_blocks_per_sm(kTruncArena);
+    const int arena = mld::trunc_arena(units, sms);
+    const int bps = mld::trunc_blocks_per_sm(arena);
     if (bps < 1) return MLD_ERR_CUDA;
     const int upb = mld::trunc_units_per_block();
     int64_t blocks1 = (int64_t)bps * sms;
@@ -881,7 +881,7 @@ mld_status decode_truncated(mld_code* C, const mld::Plan& P, const mld::SiteStep
     ta.noise_mode = noise_mode;
     ta.chi = chi;
     ta.cutoff = C->svd_cutoff;
-    ta.arena = kTruncArena;
+    ta.arena = arena;
     ta.caps = caps1;
     ta.ws = C->d_tws;
     ta.next_unit = reinterpret_cast<unsigned long long*>(ctl);
@@ -896,6 +896,7 @@ mld_status decode_truncated(mld_code* C, const mld::Plan& P, const mld::SiteStep
     const int* last_count = reinterpret_cast<const int*>(ctl + 16);
     if (pass2) {
         ta.caps = mld::kTruncLarge;
+        ta.arena = mld::kTruncArenas[2];       // few and heavy units on one block per 4 SMs
         ta.next_unit = reinterpret_cast<unsigned long long*>(ctl + 8);
         ta.in_list = C->d_ovf;
         ta.in_count = reinterpret_cast<const int*>(ctl + 16);

@@ -22,6 +22,17 @@ constexpr TruncCaps kTruncSmall{48, 192, 128 * 1024, 256 * 1024, 64 * 1024};
 constexpr TruncCaps kTruncMid{64, 256, 256 * 1024, 512 * 1024, 128 * 1024};
 constexpr TruncCaps kTruncLarge{128, 512, 1024 * 1024, 2048 * 1024, 384 * 1024};
 
+// On-chip work arena of a unit (floats): 16, 8 or 4 warps share an SM. Batches
+// that leave an SM at most 8 or 4 units get the larger ones: their time is the
+// heaviest unit's, whose large steps then stay on chip (d = 25, chi = 64, 515
+// syndromes: 130 ms with 8 warps, 153 with 16; d = 17, p = 0.17, 128 syndromes:
+// 133 ms with 4, 149 with 8, 181 with 16; under load more warps are faster:
+// d = 17, 8,192 syndromes 237 ms with 16, 279 with 8, 450 with 4).
+constexpr int kTruncArenas[3] = {3072, 6500, 13500};
+constexpr int trunc_arena(int64_t units, int sms) {
+    return kTruncArenas[units <= 4 * (int64_t)sms ? 2 : (units <= 8 * (int64_t)sms ? 1 : 0)];
+}
+
 struct TruncArgs {
     const uint64_t* dmask;           // [n][2][words]
     const float* noise;              // [n][4] or [B]
