@@ -18,10 +18,10 @@
 // their midpoint, I - Lambda is banded (bandwidth about 3d) apart from the tie
 // path's middle edge, which is ordered last as a two-row, two-column border,
 // and the sector edge's two columns are the last two of the band. One warp
-// (d <= 13) or one block of four warps (d >= 15, with look-ahead: while warps
-// 1-3 apply step k to columns k+2.., warp 0 applies it to column k+1, places
-// the entering row and takes step k+1's pivot and multipliers) eliminates
-// one matrix with partial pivoting, streaming: only the rows and
+// (d <= 15) or one block of four warps (above, with look-ahead: while warps 2
+// and 3 apply step k to columns k+2.., warp 0 applies it to column k+1 and
+// takes step k+1's pivot and multipliers, and warp 1 writes the entering row)
+// eliminates one matrix with partial pivoting, streaming: only the rows and
 // columns of the current band window are in shared memory (rows enter as the
 // elimination reaches them; a row leaves when it has been the pivot). The
 // border columns and a second copy of the two sector columns (their sector-1
@@ -242,7 +242,10 @@ struct KwArgs {
     double* flops;      // executed-flop counter (one atomic add per part)
 };
 
-// Warps per syndrome window of the look-ahead block kernel.
+// Warps per syndrome window of the look-ahead block kernel (warp 0 the pivot
+// chain, warp 1 the entering row, the others the update; 5, 6 and 8 were
+// slower: 26, 27 and 31 ms against 18 for 8,191 syndromes at d = 17, the chain
+// warps then sharing their schedulers with update warps).
 constexpr int kKwWarps = 4;
 
 // Shared memory of the one-warp kernel: the window rows (WR band slots, then
@@ -710,6 +713,24 @@ __host__ __device__ inline KwLayoutLA kw_layout_la(int WR, int RS, int n, size_t
     return L;
 }
 
+// The block kernel's complex arithmetic with its contractions written out: every
+// rounding decides pivots at the accuracy this path has, so its bits are kept
+// whatever surrounds an expression. Of the two products of a sum the first
+// is fused, or in the imaginary part the second (SECOND).
+template <bool SECOND>
+__device__ __forceinline__ float2 kw_product(float2 a, float2 b) {
+    const float re = __fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y));
+    const float im = SECOND ? __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)) : __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x));
+    return make_float2(re, im);
+}
+template <bool SECOND>
+__device__ __forceinline__ void kw_sub_product(float2& r, float2 m, float2 u) {
+    const float2 p = kw_product<SECOND>(m, u);
+    r.x = __fsub_rn(r.x, p.x);
+    r.y = __fsub_rn(r.y, p.y);
+}
+__device__ __forceinline__ float kw_norm2(float2 v) { return __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y)); }
+
 // Warp 0's part of a step, for step j (column j at position colj, logical
 // row j at map position kmodj): the pivot among rows j..j+bl, the row
 // exchange, the pivot's squared modulus into the mantissa, the multipliers
@@ -717,115 +738,108 @@ __host__ __device__ inline KwLayoutLA kw_layout_la(int WR, int RS, int n, size_t
 // the lists of buffer b, column j of those rows zeroed, their extents grown.
 // Lane l holds the rows at offsets l, l + 32, l + 64 from j (slot and column
 // j entry) from the pivot search to the multipliers; the exchange swaps two
-// of them between lanes.
-template <typename T, typename C>
-__device__ __forceinline__ void kw_la_pivot(const KwArgs& a, C* A, C* mult, int* map, int* ext, int* act, int* ctl,
-                                            int j, int colj, int kmodj, int b, int lane, T& mant, int& expo,
-                                            long long& rows_done, long long& cols_done) {
+// of them between lanes. The row at offset `entering` (-1: none) is being
+// written by warp 1: its entry of column j is `fresh`. Returns the pivot's
+// slot, its last column and the number of active rows (nact < 0: no pivot).
+struct KwStep {
+    int ps, extp, nact;
+};
+__device__ __forceinline__ KwStep kw_la_pivot(const KwArgs& a, float2* A, float2* mult, int* map, int* ext, int* act,
+                                              int* ctl, int j, int colj, int kmodj, int b, int lane, int entering,
+                                              float2 fresh, float& mant, int& expo, long long& rows_done,
+                                              long long& cols_done) {
     const unsigned FULL = 0xffffffffu;
     const int WR = a.WR, RS = a.RS, Nb = a.Nb, BR = a.WR + 1;
-    const C zero = C{T(0), T(0)};
+    const float2 zero = make_float2(0.f, 0.f);
     const int kend = (j + a.bl < Nb - 1) ? j + a.bl : Nb - 1;
     const int span = kend - j;                       // offsets 0..span
     int sl[kKwMaxChunks];
-    C vv[kKwMaxChunks];
-    T best = T(-1);
+    float2 vv[kKwMaxChunks];
+    float best = -1.f;
     int boff = 0;
+    const float2 border = lane < 2 ? A[(size_t)(BR + lane) * RS + colj] : zero;
 #pragma unroll
     for (int c = 0; c < kKwMaxChunks; ++c) {
         const int off = lane + 32 * c;
-        sl[c] = 0;
+        int mp = kmodj + off;
+        if (mp >= WR) mp -= WR;
+        sl[c] = off <= span ? map[mp] : 0;
+    }
+#pragma unroll
+    for (int c = 0; c < kKwMaxChunks; ++c) {
+        const int off = lane + 32 * c;
         vv[c] = zero;
         if (off <= span) {
-            int mp = kmodj + off;
-            if (mp >= WR) mp -= WR;
-            sl[c] = map[mp];
-            vv[c] = A[(size_t)sl[c] * RS + colj];
-            const T m2 = vv[c].x * vv[c].x + vv[c].y * vv[c].y;
+            vv[c] = off == entering ? fresh : A[(size_t)sl[c] * RS + colj];
+            const float m2 = kw_norm2(vv[c]);
             if (m2 > best) {
                 best = m2;
                 boff = off;
             }
         }
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const T ob = __shfl_xor_sync(FULL, best, o);
-        const int oo = __shfl_xor_sync(FULL, boff, o);
-        if (ob > best || (ob == best && oo < boff)) {
-            best = ob;
-            boff = oo;
-        }
-    }
-    if (!(best > T(0))) {
+    // largest, lowest offset: the bits of values >= 0 (and of -1) order as integers
+    const int top = __reduce_max_sync(FULL, __float_as_int(best));
+    boff = __reduce_min_sync(FULL, __float_as_int(best) == top ? boff : 0x7fffffff);
+    best = __int_as_float(top);
+    KwStep step = {0, 0, -1};
+    if (!(best > 0.f)) {
         if (lane == 0) ctl[b * 4 + 3] = 1;
-        return;
+        return step;
     }
+    // the pivot's slot and entry, and what the exchange of offsets 0 and boff moves
+    const int lb = boff & 31, cb = boff >> 5;
+    const float2 v_b = cb == 0 ? vv[0] : (cb == 1 ? vv[1] : vv[2]);
+    const int ps = __shfl_sync(FULL, cb == 0 ? sl[0] : (cb == 1 ? sl[1] : sl[2]), lb);
+    const float2 u = make_float2(__shfl_sync(FULL, v_b.x, lb), __shfl_sync(FULL, v_b.y, lb));
+    const int s_0 = __shfl_sync(FULL, sl[0], 0);
+    const float2 v_0 = make_float2(__shfl_sync(FULL, vv[0].x, 0), __shfl_sync(FULL, vv[0].y, 0));
+    const int extp = ext[ps];
+    const float inv2 = 1.f / best;
+    const float2 inv = make_float2(u.x * inv2, -u.y * inv2);
     if (boff != 0) {
-        // exchange offsets 0 and boff in the map and in the lanes' registers
-        const int lb = boff & 31, cb = boff >> 5;
-        const int s_b = __shfl_sync(FULL, cb == 0 ? sl[0] : (cb == 1 ? sl[1] : sl[2]), lb);
-        const C v_b = cb == 0 ? vv[0] : (cb == 1 ? vv[1] : vv[2]);
-        const T vbx = __shfl_sync(FULL, v_b.x, lb), vby = __shfl_sync(FULL, v_b.y, lb);
-        const int s_0 = __shfl_sync(FULL, sl[0], 0);
-        const T v0x = __shfl_sync(FULL, vv[0].x, 0), v0y = __shfl_sync(FULL, vv[0].y, 0);
         if (lane == 0) {
             int mp = kmodj + boff;
             if (mp >= WR) mp -= WR;
-            map[kmodj] = s_b;
+            map[kmodj] = ps;
             map[mp] = s_0;
-            sl[0] = s_b;
-            vv[0] = C{vbx, vby};
         }
         if (lane == lb) {
 #pragma unroll
             for (int c = 0; c < kKwMaxChunks; ++c)
                 if (c == cb) {
                     sl[c] = s_0;
-                    vv[c] = C{v0x, v0y};
+                    vv[c] = v_0;
                 }
         }
     }
-    const int ps = __shfl_sync(FULL, sl[0], 0);
-    const C u = C{__shfl_sync(FULL, vv[0].x, 0), __shfl_sync(FULL, vv[0].y, 0)};
-    const T inv2 = T(1) / best;
-    const C inv = C{u.x * inv2, -u.y * inv2};
-    if (lane == 0) {
-        int e;
-        mant *= best;
-        mant = sizeof(T) == 4 ? (T)frexpf((float)mant, &e) : (T)frexp((double)mant, &e);
-        expo += e;
-    }
-    const int extp = ext[ps];
     int* actb = act + b * (WR + 2);
-    C* multb = mult + b * (WR + 2);
+    float2* multb = mult + b * (WR + 2);
     int nact = 0;
     // band rows: offsets 1..span, from the registers
 #pragma unroll
     for (int c = 0; c < kKwMaxChunks; ++c) {
         const int off = lane + 32 * c;
-        const bool nz = off >= 1 && off <= span && (vv[c].x != T(0) || vv[c].y != T(0));
+        const bool nz = off >= 1 && off <= span && (vv[c].x != 0.f || vv[c].y != 0.f);
         const unsigned bal = __ballot_sync(FULL, nz);
         if (nz) {
             const int q = nact + __popc(bal & ((1u << lane) - 1u));
             const int s = sl[c];
             actb[q] = s;
-            multb[q] = C{vv[c].x * inv.x - vv[c].y * inv.y, vv[c].x * inv.y + vv[c].y * inv.x};
+            multb[q] = kw_product<false>(vv[c], inv);
             A[(size_t)s * RS + colj] = zero;
-            if (ext[s] < extp) ext[s] = extp;
+            atomicMax(&ext[s], extp);
         }
         nact += __popc(bal);
     }
     // the border rows
     {
-        C v = zero;
-        if (lane < 2) v = A[(size_t)(BR + lane) * RS + colj];
-        const bool nz = lane < 2 && (v.x != T(0) || v.y != T(0));
+        const bool nz = lane < 2 && (border.x != 0.f || border.y != 0.f);
         const unsigned bal = __ballot_sync(FULL, nz);
         if (nz) {
             const int q = nact + __popc(bal & ((1u << lane) - 1u));
             actb[q] = BR + lane;
-            multb[q] = C{v.x * inv.x - v.y * inv.y, v.x * inv.y + v.y * inv.x};
+            multb[q] = kw_product<true>(border, inv);
             A[(size_t)(BR + lane) * RS + colj] = zero;
         }
         nact += __popc(bal);
@@ -835,20 +849,39 @@ __device__ __forceinline__ void kw_la_pivot(const KwArgs& a, C* A, C* mult, int*
         ctl[b * 4 + 1] = extp;
         ctl[b * 4 + 2] = nact;
         ctl[b * 4 + 3] = 0;
-        rows_done += nact;
-        cols_done += (long long)nact * (extp - j + 4);
     }
+    // frexp of the product (the library call only outside the normal range)
+    mant *= best;
+    const uint32_t mb = __float_as_uint(mant);
+    int e = (int)(mb >> 23) - 126;
+    if (e > -126 && e < 129)
+        mant = __uint_as_float((mb & 0x7fffffu) | 0x3f000000u);
+    else
+        mant = frexpf(mant, &e);
+    expo += e;
+    rows_done += nact;
+    cols_done += (long long)nact * (extp - j + 4);
     __syncwarp();
+    step.ps = ps;
+    step.extp = extp;
+    step.nact = nact;
+    return step;
 }
 
-// ln Z of one part for both sectors, W warps per syndrome with look-ahead:
-// in step k warp 0 applies step k's update to column k+1, places the
-// entering row in the spare slot and takes step k+1's pivot and multipliers,
-// while warps 1..W-1 apply step k's update to columns k+2.. and the extra
-// columns. One block barrier per step; step k's lists are in buffer k & 1.
-template <typename T, int NT, int W>
+// ln Z of one part for both sectors, W warps per syndrome with look-ahead: in
+// step k warp 0 applies step k's update to column k+1 and takes step k+1's
+// pivot and multipliers, warp 1 writes the entering row to the spare slot, the
+// others apply step k's update to columns k+2.. and the extra columns. One
+// block barrier per step; step k's lists are in buffer k & 1. Bound: warp 0's
+// chain, 1,900 cycles a step, 1,200 of them in the pivot (2,900 with the
+// entering row on it, all four pivot-row passes run and shuffles for the
+// search); a window takes 50 KB of shared memory at d = 17, so four blocks
+// share an SM. Measured: d = 17, 8,191 syndromes 18.2 ms (30.1), d = 25, 600
+// syndromes 5.6 ms (8.5).
+template <int W>
 __device__ __forceinline__ void kw_part_la(const KwArgs& a, unsigned char* base, double out[2]) {
-    using C = typename Cplx<T>::type;
+    using T = float;
+    using C = float2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned FULL = 0xffffffffu;
     const KwLayoutLA L = kw_layout_la(a.WR, a.RS, a.n, sizeof(C));
@@ -873,10 +906,10 @@ __device__ __forceinline__ void kw_part_la(const KwArgs& a, unsigned char* base,
         kw_place_row<T, C>(a, A + (size_t)i * RS, i, j, v, v1, lane);
         if (lane == 0) ext[i] = a.ext0[i];
     }
-    // border rows (warp 0 keeps each lane's entry of both)
+    // border rows (warp 1 keeps each lane's entry of both)
     int bj[2] = {-1, -1};
     C bv[2] = {zero, zero};
-    if (warp == 0) {
+    if (warp == 1) {
         for (int t = 0; t < 2; ++t) {
             C v1;
             bj[t] = kw_fetch<T, C>(a, wt, Nb + t, lane, bv[t], v1);
@@ -895,9 +928,9 @@ __device__ __forceinline__ void kw_part_la(const KwArgs& a, unsigned char* base,
     T mant = T(1);
     int expo = 0;
     long long rows_done = 0, cols_done = 0;
-    int spare = WR;                         // the free band slot (warp 0)
-    // warp 0 reads the table entries of the row entering at step k during
-    // step k-1 (column, weight source, phase, extent), off its critical path
+    int spare = WR;                         // the free band slot (warps 0 and 1)
+    // warps 0 and 1 read the table entries of the row entering at step k
+    // during step k-1 (column, weight source, phase, extent)
     int fj = -1, fs = 0, fext = 0;
     double2 fph = make_double2(0.0, 0.0);
     auto prefetch = [&](int i) {
@@ -908,38 +941,69 @@ __device__ __forceinline__ void kw_part_la(const KwArgs& a, unsigned char* base,
             fext = a.ext0[i];
         }
     };
-    if (warp == 0) prefetch(WR);
+    if (warp < 2) prefetch(WR);
+    KwStep st = {0, 0, 0};
     if (warp == 0)
-        kw_la_pivot<T, C>(a, A, mult, map, ext, act, ctl, 0, 0, 0, 0, lane, mant, expo, rows_done, cols_done);
+        st = kw_la_pivot(a, A, mult, map, ext, act, ctl, 0, 0, 0, 0, lane, -1, zero, mant, expo, rows_done, cols_done);
     __syncthreads();
     bool dead = false;
     int colk = 0, kmod = 0;    // k mod WC, k mod WR
+    int colin = WR % WC;       // (k + WR) mod WC
     for (int k = 0; k < Nb - 2; ++k) {
         const int b = k & 1;
-        if (ctl[b * 4 + 3]) {
-            dead = true;
-            break;
+        if (warp == 0) {
+            if (st.nact < 0) dead = true;
+        } else {
+            dead = ctl[b * 4 + 3] != 0;
+            st.ps = ctl[b * 4 + 0];
+            st.extp = ctl[b * 4 + 1];
+            st.nact = ctl[b * 4 + 2];
         }
-        const int ps = ctl[b * 4 + 0], extp = ctl[b * 4 + 1], nact = ctl[b * 4 + 2];
+        if (dead) break;
+        const int ps = st.ps, extp = st.extp, nact = st.nact;
         const int* actb = act + b * (WR + 2);
         const C* multb = mult + b * (WR + 2);
         const C* P = A + (size_t)ps * RS;
         const int colk1 = colk + 1 == WC ? 0 : colk + 1;
         const int kmod1 = kmod + 1 == WR ? 0 : kmod + 1;
+        // row k + WR enters in the spare slot (its map position is k's); the
+        // pivot's slot becomes the spare
+        const int rin = k + WR;
         if (warp == 0) {
             // step k's update of column k+1
             const C u1 = k + 1 <= extp ? P[colk1] : zero;
             for (int q = lane; q < nact; q += 32) {
                 C* R = A + (size_t)actb[q] * RS;
                 C r = R[colk1];
-                kw_axpy<C, T>(r, multb[q], u1);
+                kw_sub_product<true>(r, multb[q], u1);
                 R[colk1] = r;
             }
-            // row k + WR enters in the spare slot (its map position is
-            // k's); the pivot's slot becomes the spare
-            const int rin = k + WR;
+            // the entering row's entry of column k+1 (its first column at the least)
+            C fresh = zero;
+            int entering = -1;
             if (rin < Nb) {
-                const int j = fj, ext_in = fext;
+                const T w = fs >= 0 ? wt[fs] : T(1);
+                const C v = C{-w * (T)fph.x, -w * (T)fph.y};
+                const unsigned has = __ballot_sync(FULL, fj == k + 1);
+                if (has) {
+                    const int l = __ffs(has) - 1;
+                    fresh = C{__shfl_sync(FULL, v.x, l), __shfl_sync(FULL, v.y, l)};
+                }
+                entering = a.bl;
+                if (lane == 0) {
+                    ext[spare] = fext;
+                    map[kmod] = spare;
+                }
+                prefetch(rin + 1);
+                spare = ps;
+            }
+            __syncwarp();
+            if (k + 1 < Nb - 2)
+                st = kw_la_pivot(a, A, mult, map, ext, act, ctl, k + 1, colk1, kmod1, b ^ 1, lane, entering, fresh,
+                                 mant, expo, rows_done, cols_done);
+        } else if (warp == 1) {
+            if (rin < Nb) {
+                const int j = fj;
                 const T w = fs >= 0 ? wt[fs] : T(1);
                 const C v = C{-w * (T)fph.x, -w * (T)fph.y};
                 const C v1 = fs == -2 ? C{(T)fph.x, (T)fph.y} : v;
@@ -947,10 +1011,19 @@ __device__ __forceinline__ void kw_part_la(const KwArgs& a, unsigned char* base,
                 C* R = A + (size_t)spare * RS;
                 for (int i = lane; i < RS; i += 32) R[i] = zero;
                 __syncwarp();
-                kw_place_row<T, C>(a, R, rin, j, v, v1, lane);
+                // (its entry of column k+1 goes to warp 0 directly: that column
+                // of the row is eliminated, or the row the pivot, this step)
+                if (j >= Nb) {
+                    R[WC + (j - Nb)] = v;
+                } else if (j >= 0 && j != k + 1) {
+                    int p = colin + (j - rin);           // |j - rin| <= bl, bu < WC
+                    p = p < 0 ? p + WC : (p >= WC ? p - WC : p);
+                    R[p] = v;
+                    if (j >= Nb - 2) R[WC + 2 + (j - (Nb - 2))] = v1;
+                }
                 if (lane == 0) {
-                    ext[spare] = ext_in;
-                    map[kmod] = spare;
+                    R[colin].x = T(1);
+                    if (rin >= Nb - 2) R[WC + 2 + (rin - (Nb - 2))].x = T(1);
                 }
                 spare = ps;
             }
@@ -959,46 +1032,51 @@ __device__ __forceinline__ void kw_part_la(const KwArgs& a, unsigned char* base,
 #pragma unroll
             for (int t = 0; t < 2; ++t)
                 if (bj[t] == jn && jn < Nb) A[(size_t)(BR + t) * RS + colk] = bv[t];
-            __syncwarp();
-            if (k + 1 < Nb - 2)
-                kw_la_pivot<T, C>(a, A, mult, map, ext, act, ctl, k + 1, colk1, kmod1, b ^ 1, lane, mant, expo,
-                                  rows_done, cols_done);
         } else {
-            // step k's update of columns k+2..extp and the four extra columns
-            C U[NT];
-            int pc[NT];
-#pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                const int c = k + 1 + lane + 32 * t;
-                int p = colk + 1 + lane + 32 * t;
+            // step k's update of columns k+2..extp and the four extra columns,
+            // 32 of them at a time, a lane each: pivot rows reach some 34
+            // columns (four fixed passes per row, empty lanes and all, took
+            // 2.1 M warp instructions a syndrome at d = 17)
+            const int own = extp - (k + 1) > 0 ? extp - (k + 1) : 0, total = own + 4;
+            for (int c0 = 0; c0 < total; c0 += 32) {
+                const int c = c0 + lane;
+                int p = colk + 2 + c;
                 if (p >= WC) p -= WC;
-                pc[t] = (c >= k + 2 && c <= extp) ? p : -1;
-                U[t] = pc[t] >= 0 ? P[p] : zero;
-            }
-            const C Ux = lane < 4 ? P[WC + lane] : zero;
-            for (int q = warp - 1; q < nact; q += W - 1) {
-                C* R = A + (size_t)actb[q] * RS;
-                const C m = multb[q];
-                C r[NT], rx;
+                if (c >= own) p = WC + (c - own);
+                const bool in = c < total;
+                const C u = in ? P[p] : zero;
+                int q = warp - 2;
+                for (; q + 3 * (W - 2) < nact; q += 4 * (W - 2)) {
+                    C* R[4];
+                    C m[4], r[4];
 #pragma unroll
-                for (int t = 0; t < NT; ++t)
-                    if (pc[t] >= 0) r[t] = R[pc[t]];
-                if (lane < 4) rx = R[WC + lane];
-#pragma unroll
-                for (int t = 0; t < NT; ++t)
-                    if (pc[t] >= 0) {
-                        kw_axpy<C, T>(r[t], m, U[t]);
-                        R[pc[t]] = r[t];
+                    for (int t = 0; t < 4; ++t) {
+                        R[t] = A + (size_t)actb[q + t * (W - 2)] * RS + p;
+                        m[t] = multb[q + t * (W - 2)];
+                        if (in) r[t] = *R[t];
                     }
-                if (lane < 4) {
-                    kw_axpy<C, T>(rx, m, Ux);
-                    R[WC + lane] = rx;
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        if (in) {
+                            kw_sub_product<false>(r[t], m[t], u);
+                            *R[t] = r[t];
+                        }
+                }
+                for (; q < nact; q += W - 2) {
+                    C* R = A + (size_t)actb[q] * RS + p;
+                    const C m = multb[q];
+                    if (in) {
+                        C r = *R;
+                        kw_sub_product<false>(r, m, u);
+                        *R = r;
+                    }
                 }
             }
         }
         __syncthreads();
         colk = colk1;
         kmod = kmod1;
+        colin = colin + 1 == WC ? 0 : colin + 1;
     }
 
     if (warp == 0) {
@@ -1024,7 +1102,7 @@ __device__ __forceinline__ void kw_part_la(const KwArgs& a, unsigned char* base,
 // One block of W warps per syndrome with the look-ahead schedule (d >= 15),
 // persistent over the batch; the same steps as kw_decode_warp_kernel.
 template <typename T, int NT>
-__global__ void __launch_bounds__(32 * kKwWarps) kw_decode_la_kernel(KwArgs a) {
+__global__ void __launch_bounds__(32 * kKwWarps, 4) kw_decode_la_kernel(KwArgs a) {
     constexpr int W = kKwWarps;
     extern __shared__ __align__(16) unsigned char kw_smem[];
     using C = typename Cplx<T>::type;
@@ -1051,7 +1129,7 @@ __global__ void __launch_bounds__(32 * kKwWarps) kw_decode_la_kernel(KwArgs a) {
         }
         zany = __syncthreads_or(zany);
         double lx[2], lz[2];
-        kw_part_la<T, NT, W>(a, base, lx);
+        kw_part_la<W>(a, base, lx);
         if (a.pz) {
             for (int qt = tid; qt < n; qt += 32 * W) {
                 const int q = a.zmap[qt];
@@ -1063,7 +1141,7 @@ __global__ void __launch_bounds__(32 * kKwWarps) kw_decode_la_kernel(KwArgs a) {
                 wt[qt] = (z ? T(-1) : T(1)) * (T(1) - T(2) * (T)p);
             }
             __syncthreads();
-            kw_part_la<T, NT, W>(a, base, lz);
+            kw_part_la<W>(a, base, lz);
         } else {
             lz[0] = zany ? -INFINITY : 0.0;
             lz[1] = -INFINITY;
