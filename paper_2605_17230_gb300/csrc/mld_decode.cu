@@ -803,12 +803,11 @@ mld_status grow(T** buf, size_t* have, size_t bytes) {
     return MLD_OK;
 }
 
-// Truncating chi: the rank-adaptive kernel (one warp per unit) over all units
-// on every resident warp, with the smallest slice capacities that hold bonds
-// of chi (bond 48, 64 or 128: 2.25, 4.5 or 17.8 MB per resident warp), or
+// Truncating chi: the rank-adaptive kernel over all units, with the smallest slice capacities that hold bonds
+// of chi (bond 48, 64 or 128: 2.25, 4.5 or 17.8 MB per resident unit), or
 // smaller ones if that workspace cannot be allocated or the code's cap is
 // lower; the units it hands back go to a second pass of the same kernel with
-// the bond-128 capacities on one block of warps per 4 SMs, and what that
+// the bond-128 capacities, a unit per SM, and what that
 // hands back (bonds above 128) to the fixed-shape kernel in global-workspace
 // mode. (A unit handed back restarts from its first column on few warps, so
 // the first pass's capacities decide how long that tail is: at d=25 with
@@ -831,11 +830,12 @@ mld_status decode_truncated(mld_code* C, const mld::Plan& P, const mld::SiteStep
     const int arena = mld::trunc_arena(units, sms);
     const int bps = mld::trunc_blocks_per_sm(arena);
     if (bps < 1) return MLD_ERR_CUDA;
-    const int upb = mld::trunc_units_per_block();
+    const int upb = mld::trunc_units_per_block(arena);
     int64_t blocks1 = (int64_t)bps * sms;
     if (blocks1 > (units + upb - 1) / upb) blocks1 = (units + upb - 1) / upb;
-    int64_t blocks2 = (sms + 3) / 4;
-    const size_t ws2 = (size_t)blocks2 * upb * mld::kTruncLarge.slice();
+    const int upb2 = mld::trunc_units_per_block(mld::kTruncArenas[2]);
+    const int64_t blocks2 = (sms + 3) / 4 * (4 / upb2);         // a unit per SM
+    const size_t ws2 = (size_t)blocks2 * upb2 * mld::kTruncLarge.slice();
     // first-pass capacities: the smallest that hold bonds of chi (at most the
     // cap set by mld_code_set_truncation_workspace); if that workspace cannot
     // be allocated, the next smaller ones

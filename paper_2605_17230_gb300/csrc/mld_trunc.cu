@@ -19,11 +19,14 @@
 // preconditioning: the rows of a pivoted R are nearly orthogonal, so few
 // sweeps settle) over r' columns instead of all of T.
 //
-// One warp owns one (syndrome, l_Z) unit (both l_X classes: the X_L string
+// One warp sweeps one (syndrome, l_Z) unit (both l_X classes: the X_L string
 // sits on column d-1, columns 0..d-2 are swept once and the last column once
 // per l_X from the state they leave); warps are persistent and take units
 // from a device queue. The matrices are small (tens of rows), so a warp per
-// unit keeps every step warp-synchronous and many units resident per SM.
+// unit keeps every step warp-synchronous and many units resident per SM. In
+// batches that leave warps idle a unit has a team of two or four: the others
+// take their share of the loops over more than 32 columns (MPO products,
+// reflections, applications of Q), which are the heavy units' steps.
 // Each site step lays its buffers out from its actual shapes in the warp's
 // shared-memory arena: the incoming carry at one end, the outgoing carry at
 // the other (ends alternate from step to step, so a carry is never moved),
@@ -42,15 +45,16 @@
 // other components (a cutoff 10% off moves posteriors by 4e-5).
 //
 // Bound: instruction fetch under load (16 warps an SM at different places of
-// an 78 KB program; 0.3 instructions a clock and SM), the latency of the
+// a 78 KB program; 0.3 instructions a clock and SM), the latency of the
 // heaviest unit's chain in small batches (a unit takes up to six times the
 // mean, most of it in the few per cent of steps that spill). Hence loops are
 // not unrolled beyond loading four rows ahead of their stores, copies run
 // over flattened indices, arg-max and maximum are integer reductions, and
-// small batches get larger arenas on fewer warps. Measured on GB300: d = 17,
-// chi = 32, 2,048 syndromes 93 ms (178 with loops unrolled by the compiler,
+// small batches get larger arenas and teams. Measured on GB300: d = 17,
+// chi = 32, 2,048 syndromes 91 ms (178 with loops unrolled by the compiler,
 // spilled steps walking global columns), 8,192 syndromes 237 ms (449); d = 25,
-// chi = 64, 515 syndromes 130 ms (321).
+// chi = 64, 515 syndromes 114 ms (130 without teams; 321); d = 17, p = 0.17, 32
+// syndromes 65 ms (89 without teams), one easy syndrome at d = 19 23.0 (24.1).
 //
 // Matrices on chip are column-major with odd leading dimensions (lanes walking
 // one column each hit distinct banks), in the spill arena row-major (the lanes
@@ -59,13 +63,15 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "mld_internal.h"
 #include "mld_trunc.h"
 
 namespace mld {
 namespace trunc {
 
-constexpr int kWarpsPerBlock = 4;         // units per block
+constexpr int kWarpsPerBlock = 4;         // one, two or four units
 constexpr int kMaxSweeps = 40;
 constexpr float kTol = 1.0e-5f;           // pair orthogonality threshold (as the fixed-shape kernel)
 constexpr float kNoise = 1.0e-8f;         // rotations moving less than this of the block are skipped
@@ -117,24 +123,80 @@ __device__ __forceinline__ int odd(int k) { return k | 1; }
 // alias).
 constexpr int kAhead = 4;
 
-// Householder QR with column pivoting, in place, of a K x N matrix (element
-// (r, c) at r rs + c cs). Step j swaps the column of largest remaining
-// norm into place, forms its reflector (R on and above the diagonal, the tail
-// below it with v_j[j] = 1 implied, tau[j]) and applies it to the later
-// columns; piv[j] is the original index of the column now at j. It stops once
-// every remaining column norm is at most thr_rel times the largest initial
-// one (or after min(K, N, maxr) steps) and returns the step count r. The
-// reflector is formed across the warp's lanes; the later columns are updated
-// one per lane (their row loops run serially, with no cross-lane reduction).
-// The reflector norm is taken of the column scaled by a power of two near its
-// maximum (a column far below the matrix's largest entries would lose its
-// squares to underflow).
-__device__ __noinline__ int qrcp(float* M, int K, int rs, int cs, int N, float* tau, int* piv, float* nrm,
-                                 float thr_rel, int maxr, unsigned long long* fl) {
-    const int lane = threadIdx.x & 31;
+// A pointer into shared memory as a 32-bit index: loads and stores through it
+// are shared-memory instructions with 32-bit addresses. A float* that may point
+// to either memory costs 64-bit address arithmetic for every element, more
+// instructions than the arithmetic itself.
+struct Sh {
+    int o;
+    __device__ __forceinline__ float& operator[](int i) const {
+        extern __shared__ __align__(16) unsigned char smem_raw[];
+        return reinterpret_cast<float*>(smem_raw)[o + i];
+    }
+    __device__ __forceinline__ float& operator*() const { return (*this)[0]; }
+    __device__ __forceinline__ Sh operator+(int i) const { return Sh{o + i}; }
+    __device__ __forceinline__ Sh& operator+=(int i) { o += i; return *this; }
+    __device__ __forceinline__ Sh& operator++() { ++o; return *this; }
+};
+__device__ __forceinline__ Sh shared_of(const float* p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    return Sh{(int)(p - reinterpret_cast<const float*>(smem_raw))};
+}
+// Row stride of a matrix on chip: 1.
+template <class P>
+constexpr bool kChip = std::is_same_v<P, Sh>;
+// With one warp a unit and sixteen units an SM the second copy of each loop
+// costs more (instruction fetch) than its addresses: one copy there.
+template <int T>
+using ChipPtr = std::conditional_t<(T > 1), Sh, float*>;
+
+// A unit's team is T warps (T = 1, 2, 4). Warp 0 runs the sweep; the others wait
+// at the team's barrier for a loop over columns or entries that is worth
+// sharing, run their part of it and meet warp 0 there again. Each
+// column or entry is computed by one lane or lane group as warp 0 alone would,
+// so the bits do not depend on T.
+enum JobKind { kQuit, kApply, kNorms, kUpdate, kApplyQ, kScale };
+struct Job {
+    int kind;
+    int chip;                             // which matrices are on chip
+    float part[4];                        // maxima of the warps' parts
+    const float *C, *A, *wq, *V0, *tau0, *V1, *tau1;
+    float *M, *nrm;
+    int K, N, rs, cs, j, ncolA, Dl, Dr, ldC, pam, par, bp, i, rsplit, nr0, nr1, split, vrs, vcs;
+    float f;
+};
+
+// The barrier of this thread's team (0 is the block's).
+template <int T>
+__device__ __forceinline__ void team_barrier() {
+    __syncwarp();
+    static_assert(kWarpsPerBlock == 4, "two teams of two warps or one of four");
+    if (T == 4 || threadIdx.x < 64) asm volatile("barrier.sync 1, %0;" ::"n"(32 * T) : "memory");
+    else asm volatile("barrier.sync 2, %0;" ::"n"(32 * T) : "memory");
+}
+
+// Elements lane, lane + 32, ... (step apart), four loads ahead of their stores.
+__device__ __forceinline__ void copy_floats(float* dst, const float* src, int n, int first, int step) {
+    int e = first;
 #pragma unroll 1
-    for (int c = lane; c < N; c += 32) {
-        const float* col = M + c * cs;
+    for (; e + 3 * step < n; e += 4 * step) {
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = src[e + u * step];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) dst[e + u * step] = x[u];
+    }
+#pragma unroll 1
+    for (; e < n; e += step) dst[e] = src[e];
+}
+
+// Column norms and the identity permutation: columns of warp w of nw.
+template <class P>
+__device__ __forceinline__ void column_norms(P M, int K, int rs_, int cs, int N, float* nrm, int w, int nw) {
+    const int rs = kChip<P> ? 1 : rs_;
+#pragma unroll 1
+    for (int c = 32 * w + (threadIdx.x & 31); c < N; c += 32 * nw) {
+        const P col = M + c * cs;
         float s = 0.f;
         int r = 0;
 #pragma unroll 1
@@ -148,8 +210,125 @@ __device__ __noinline__ int qrcp(float* M, int K, int rs, int cs, int N, float* 
 #pragma unroll 1
         for (; r < K; ++r) s = fmaf(col[r * rs], col[r * rs], s);
         nrm[c] = sqrtf(s);
-        piv[c] = c;
     }
+}
+
+// H_j on columns j+1 .. N-1 and their norms below row j: a group of G
+// lanes per column (G the largest power of two with (N-1-j) G <= 32),
+// the rows dealt round-robin over the group, the dot product and the
+// norm summed across it by shuffles. Columns of warp w of nw.
+template <class P>
+__device__ __forceinline__ void reflect_columns(P M, int K, int rs_, int cs, int N, float* nrm, int j, float tj,
+                                                int w_, int nw) {
+    const int lane = threadIdx.x & 31, rs = kChip<P> ? 1 : rs_;
+    const P vj = M + j * cs;
+    const int rem = N - 1 - j, sh = group_shift(rem), G = 1 << sh, gs = rs << sh;
+    const int groups = 32 >> sh, grp = lane >> sh, g = lane & (G - 1);
+#pragma unroll 1
+    for (int base = j + 1 + w_ * groups; base < N; base += nw * groups) {
+        const int cc = base + grp;
+        const bool act = cc < N;
+        const P col = M + (act ? cc : j) * cs;
+        const int rows = (K - j - 1 - g + G - 1) >> sh;       // this lane's rows j+1+g, +G, ..
+        const P v0 = vj + (j + 1 + g) * rs;
+        const P x0p = col + (j + 1 + g) * rs;
+        float w = 0.f;
+        if (act && tj != 0.f) {
+            if (g == 0) w = col[j * rs];
+            P vp = v0, xp = x0p;
+            int m = rows;
+#pragma unroll 1
+            for (; m >= kAhead; m -= kAhead) {
+                float v[kAhead], x[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    v[u] = vp[u * gs];
+                    x[u] = xp[u * gs];
+                }
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) w = fmaf(v[u], x[u], w);
+                vp += kAhead * gs;
+                xp += kAhead * gs;
+            }
+#pragma unroll 1
+            for (; m > 0; --m, vp += gs, xp += gs) w = fmaf(*vp, *xp, w);
+        }
+#pragma unroll 1
+        for (int o = G >> 1; o > 0; o >>= 1) w += __shfl_xor_sync(kFull, w, o);
+        float s = 0.f;
+        if (act) {
+            if (tj != 0.f) {
+                w *= tj;
+                if (g == 0) col[j * rs] -= w;
+            }
+            P vp = v0, xp = x0p;
+            int m = rows;
+#pragma unroll 1
+            for (; m >= kAhead; m -= kAhead) {
+                float v[kAhead], x[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    v[u] = vp[u * gs];
+                    x[u] = xp[u * gs];
+                }
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    if (tj != 0.f) x[u] = fmaf(-v[u], w, x[u]);
+                    xp[u * gs] = x[u];
+                    s = fmaf(x[u], x[u], s);
+                }
+                vp += kAhead * gs;
+                xp += kAhead * gs;
+            }
+#pragma unroll 1
+            for (; m > 0; --m, vp += gs, xp += gs) {
+                const float x = tj != 0.f ? fmaf(-*vp, w, *xp) : *xp;
+                *xp = x;
+                s = fmaf(x, x, s);
+            }
+        }
+#pragma unroll 1
+        for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+        if (act && g == 0) nrm[cc] = sqrtf(s);
+    }
+}
+template <int T, class P>
+__device__ __noinline__ void reflect_columns_team(P M, int K, int rs, int cs, int N, float* nrm, int j, float tj,
+                                                  int w, int nw) {
+    reflect_columns(M, K, rs, cs, N, nrm, j, tj, w, nw);
+}
+
+// Householder QR with column pivoting, in place, of a K x N matrix (element
+// (r, c) at r rs + c cs). Step j swaps the column of largest remaining
+// norm into place, forms its reflector (R on and above the diagonal, the tail
+// below it with v_j[j] = 1 implied, tau[j]) and applies it to the later
+// columns; piv[j] is the original index of the column now at j. It stops once
+// every remaining column norm is at most thr_rel times the largest initial
+// one (or after min(K, N, maxr) steps) and returns the step count r. The
+// reflector is formed across the warp's lanes; the later columns are updated
+// one per lane (their row loops run serially, with no cross-lane reduction).
+// The reflector norm is taken of the column scaled by a power of two near its
+// maximum (a column far below the matrix's largest entries would lose its
+// squares to underflow).
+template <int T, class P>
+__device__ __noinline__ int qrcp(float* Mg, int K, int rs_, int cs, int N, float* tau, int* piv, float* nrm,
+                                 float thr_rel, int maxr, unsigned long long* fl, Job* job) {
+    const int lane = threadIdx.x & 31, rs = kChip<P> ? 1 : rs_;
+    P M;
+    if constexpr (kChip<P>) M = shared_of(Mg);
+    else M = Mg;
+    const bool many = T > 1 && N > 32;
+    if (many) {
+        if (lane == 0) {
+            job->kind = kNorms;
+            job->chip = kChip<P>; job->M = Mg; job->K = K; job->rs = rs; job->cs = cs; job->N = N; job->nrm = nrm;
+        }
+        team_barrier<T>();
+    }
+    column_norms(M, K, rs, cs, N, nrm, 0, many ? T : 1);
+#pragma unroll 1
+    for (int c = lane; c < N; c += 32) piv[c] = c;
+    if (many) team_barrier<T>();
     __syncwarp();
     float thr = 0.f;
 #pragma unroll 1
@@ -173,9 +352,9 @@ __device__ __noinline__ int qrcp(float* M, int K, int rs, int cs, int N, float* 
         best = __int_as_float(top);
         if (!(best > thr && best > 0.f)) break;
         r = j + 1;
-        float* vj = M + j * cs;
+        const P vj = M + j * cs;
         if (p != j) {
-            float* cp = M + p * cs;
+            const P cp = M + p * cs;
 #pragma unroll 1
             for (int rr = lane; rr < K; rr += 32) {
                 const float t = vj[rr * rs];
@@ -215,79 +394,21 @@ __device__ __noinline__ int qrcp(float* M, int K, int rs, int cs, int N, float* 
         }
         if (lane == 0) { vj[j * rs] = beta; tau[j] = tj; }
         __syncwarp();
-        // H_j on columns j+1 .. N-1 and their norms below row j: a group of G
-        // lanes per column (G the largest power of two with (N-1-j) G <= 32),
-        // the rows dealt round-robin over the group, the dot product and the
-        // norm summed across it by shuffles
-        const int rem = N - 1 - j, sh = group_shift(rem), G = 1 << sh, gs = rs << sh;
-        const int groups = 32 >> sh, grp = lane >> sh, g = lane & (G - 1);
-#pragma unroll 1
-        for (int base = j + 1; base < N; base += groups) {
-            const int cc = base + grp;
-            const bool act = cc < N;
-            float* col = M + (act ? cc : j) * cs;
-            const int rows = (K - j - 1 - g + G - 1) >> sh;       // this lane's rows j+1+g, +G, ..
-            const float* v0 = vj + (j + 1 + g) * rs;
-            float* x0p = col + (j + 1 + g) * rs;
-            float w = 0.f;
-            if (act && tj != 0.f) {
-                if (g == 0) w = col[j * rs];
-                const float *vp = v0, *xp = x0p;
-                int m = rows;
-#pragma unroll 1
-                for (; m >= kAhead; m -= kAhead) {
-                    float v[kAhead], x[kAhead];
-#pragma unroll
-                    for (int u = 0; u < kAhead; ++u) {
-                        v[u] = vp[u * gs];
-                        x[u] = xp[u * gs];
-                    }
-#pragma unroll
-                    for (int u = 0; u < kAhead; ++u) w = fmaf(v[u], x[u], w);
-                    vp += kAhead * gs;
-                    xp += kAhead * gs;
-                }
-#pragma unroll 1
-                for (; m > 0; --m, vp += gs, xp += gs) w = fmaf(*vp, *xp, w);
+        // H_j on the later columns and their norms
+        const bool wide = T > 1 && N - 1 - j > 32;
+        if (wide) {
+            if (lane == 0) {
+                job->kind = kUpdate;
+                job->chip = kChip<P>; job->M = Mg; job->K = K; job->rs = rs; job->cs = cs; job->N = N; job->nrm = nrm;
+                job->j = j; job->f = tj;
             }
-#pragma unroll 1
-            for (int o = G >> 1; o > 0; o >>= 1) w += __shfl_xor_sync(kFull, w, o);
-            float s = 0.f;
-            if (act) {
-                if (tj != 0.f) {
-                    w *= tj;
-                    if (g == 0) col[j * rs] -= w;
-                }
-                const float* vp = v0;
-                float* xp = x0p;
-                int m = rows;
-#pragma unroll 1
-                for (; m >= kAhead; m -= kAhead) {
-                    float v[kAhead], x[kAhead];
-#pragma unroll
-                    for (int u = 0; u < kAhead; ++u) {
-                        v[u] = vp[u * gs];
-                        x[u] = xp[u * gs];
-                    }
-#pragma unroll
-                    for (int u = 0; u < kAhead; ++u) {
-                        if (tj != 0.f) x[u] = fmaf(-v[u], w, x[u]);
-                        xp[u * gs] = x[u];
-                        s = fmaf(x[u], x[u], s);
-                    }
-                    vp += kAhead * gs;
-                    xp += kAhead * gs;
-                }
-#pragma unroll 1
-                for (; m > 0; --m, vp += gs, xp += gs) {
-                    const float x = tj != 0.f ? fmaf(-*vp, w, *xp) : *xp;
-                    *xp = x;
-                    s = fmaf(x, x, s);
-                }
-            }
-#pragma unroll 1
-            for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-            if (act && g == 0) nrm[cc] = sqrtf(s);
+            team_barrier<T>();
+        }
+        if (wide) {
+            reflect_columns_team<T, P>(M, K, rs, cs, N, nrm, j, tj, 0, T);
+            team_barrier<T>();
+        } else {
+            reflect_columns(M, K, rs, cs, N, nrm, j, tj, 0, 1);
         }
         __syncwarp();
         flops += 3ULL * (K - j) + 6ULL * (K - j) * (N - 1 - j);
@@ -301,23 +422,25 @@ __device__ __noinline__ int qrcp(float* M, int K, int rs, int cs, int N, float* 
 // v_j below row j) and tau. Columns n < split use set 0 (V0, tau0, nr0), the
 // others set 1. A group of G lanes per column (G the largest power of two
 // with ncols G <= 32), the rows dealt round-robin over the group and each
-// reflector's dot product summed across it by shuffles.
-__device__ __noinline__ void apply_q(const float* V0, const float* tau0, int nr0, const float* V1,
-                                     const float* tau1, int nr1, int split, int vrs, int vcs, int K, float* Y,
-                                     int yrs, int ycs, int ncols, unsigned long long* fl) {
-    const int lane = threadIdx.x & 31;
+// reflector's dot product summed across it by shuffles. Columns of warp w_ of
+// nw.
+template <class PV, class PY>
+__device__ __noinline__ void apply_q(PV V0, const float* tau0, int nr0, PV V1,
+                                     const float* tau1, int nr1, int split, int vrs_, int vcs, int K, PY Y,
+                                     int yrs_, int ycs, int ncols, int w_, int nw) {
+    const int lane = threadIdx.x & 31, vrs = kChip<PY> ? 1 : vrs_, yrs = kChip<PY> ? 1 : yrs_;
     const int sh = group_shift(ncols), G = 1 << sh, gv = vrs << sh, gy = yrs << sh;
     const int groups = 32 >> sh, grp = lane >> sh, g = lane & (G - 1);
     const int nrmax = nr0 > nr1 ? nr0 : nr1;
 #pragma unroll 1
-    for (int base = 0; base < ncols; base += groups) {
+    for (int base = w_ * groups; base < ncols; base += nw * groups) {
         const int n = base + grp;
         const bool act = n < ncols;
         const bool s1 = n >= split;
-        const float* Vs = s1 ? V1 : V0;
+        const PV Vs = s1 ? V1 : V0;
         const float* ts = s1 ? tau1 : tau0;
         const int nr = act ? (s1 ? nr1 : nr0) : 0;
-        float* y = Y + (act ? n : 0) * ycs;
+        const PY y = Y + (act ? n : 0) * ycs;
         // every lane runs nrmax steps so that the group shuffles stay uniform;
         // lane g owns the rows r = g (mod G) in every step, so no lane reads
         // another's writes (v_j[j] = 1 is implied)
@@ -325,13 +448,14 @@ __device__ __noinline__ void apply_q(const float* V0, const float* tau0, int nr0
         for (int j = nrmax - 1; j >= 0; --j) {
             const bool on = j < nr && ts[j] != 0.f;
             const int r0 = j + ((g - j) & (G - 1));
-            const float* v0 = Vs + j * vcs + r0 * vrs;
-            float* y0 = y + r0 * yrs;
+            const PV v0 = Vs + j * vcs + r0 * vrs;
+            const PY y0 = y + r0 * yrs;
             const int rows = (K - r0 + G - 1) >> sh;
             const bool diag = r0 == j;                    // the first of this lane's rows is row j
             float w = 0.f;
             if (on) {
-                const float *vp = v0, *yp = y0;
+                PV vp = v0;
+                PY yp = y0;
                 int m = rows;
                 if (diag && m > 0) {
                     w = fmaf(1.f, *yp, w);
@@ -359,8 +483,8 @@ __device__ __noinline__ void apply_q(const float* V0, const float* tau0, int nr0
             for (int o = G >> 1; o > 0; o >>= 1) w += __shfl_xor_sync(kFull, w, o);
             if (on) {
                 w *= ts[j];
-                const float* vp = v0;
-                float* yp = y0;
+                PV vp = v0;
+                PY yp = y0;
                 int m = rows;
                 if (diag && m > 0) {
                     *yp = fmaf(-1.f, w, *yp);
@@ -386,6 +510,41 @@ __device__ __noinline__ void apply_q(const float* V0, const float* tau0, int nr0
             }
         }
     }
+    __syncwarp();
+}
+
+// apply_q where the matrices are: bit 0 of `chip`, Y on chip (and V's row
+// stride 1); bit 1, V too.
+template <int T>
+__device__ __forceinline__ void apply_q_at(int chip, const float* V0, const float* tau0, int nr0, const float* V1,
+                                           const float* tau1, int nr1, int split, int vrs, int vcs, int K, float* Y,
+                                           int yrs, int ycs, int ncols, int w, int nw) {
+    if (T > 1 && chip == 3)
+        apply_q<Sh, Sh>(shared_of(V0), tau0, nr0, shared_of(V1), tau1, nr1, split, 1, vcs, K, shared_of(Y), 1, ycs,
+                        ncols, w, nw);
+    else if (T > 1 && chip == 1)
+        apply_q<const float*, Sh>(V0, tau0, nr0, V1, tau1, nr1, split, 1, vcs, K, shared_of(Y), 1, ycs, ncols, w, nw);
+    else
+        apply_q<const float*, float*>(V0, tau0, nr0, V1, tau1, nr1, split, vrs, vcs, K, Y, yrs, ycs, ncols, w, nw);
+}
+template <int T>
+__device__ __forceinline__ void apply_q_team(int chip, const float* V0, const float* tau0, int nr0, const float* V1,
+                                             const float* tau1, int nr1, int split, int vrs, int vcs, int K, float* Y,
+                                             int yrs, int ycs, int ncols, unsigned long long* fl, Job* job) {
+    const int lane = threadIdx.x & 31;
+    const bool wide = T > 1 && ncols > 32;
+    if (wide) {
+        if (lane == 0) {
+            job->kind = kApplyQ;
+            job->chip = chip;
+            job->V0 = V0; job->tau0 = tau0; job->nr0 = nr0; job->V1 = V1; job->tau1 = tau1; job->nr1 = nr1;
+            job->split = split; job->vrs = vrs; job->vcs = vcs; job->K = K; job->M = Y; job->rs = yrs;
+            job->cs = ycs; job->N = ncols;
+        }
+        team_barrier<T>();
+    }
+    apply_q_at<T>(chip, V0, tau0, nr0, V1, tau1, nr1, split, vrs, vcs, K, Y, yrs, ycs, ncols, 0, wide ? T : 1);
+    if (wide) team_barrier<T>();
     if (lane == 0) {
         // sum_j 4 (K - j) over nr reflectors, per column
         const unsigned long long f0 = 2ULL * nr0 * (2 * K - nr0 + 1), f1 = 2ULL * nr1 * (2 * K - nr1 + 1);
@@ -395,8 +554,110 @@ __device__ __noinline__ void apply_q(const float* V0, const float* tau0, int nr0
     __syncwarp();
 }
 
+// M^{b'}[kappa][col] = sum_a w(a, a', beta(kappa), b') sum_l C[kappa][a Dl + l] A[l][col]
+// (qubit (i-1, c)), the entries of warp w_ of nw; returns this lane's largest
+// modulus. Four columns of one row at a time: one load of C for four products,
+// and four chains to overlap.
+template <class P, class PC>
+__device__ __forceinline__ float mpo_apply(const Job& a, PC C, PC A, P M, int w_, int nw) {
+    const float* wq = a.wq;
+    const int K = a.K, ncol = a.N, rsM = kChip<P> ? 1 : a.rs, csM = a.cs, ncolA = a.ncolA, Dl = a.Dl, Dr = a.Dr, ldC = a.ldC,
+              pam = a.pam, par = a.par, bp = a.bp, i = a.i, rsplit = a.rsplit;
+    const int quads = (ncol + 3) >> 2;
+    const FDiv dK(K);
+    float mx = 0.f;
+#pragma unroll 1
+    for (int e = 32 * w_ + (threadIdx.x & 31); e < K * quads; e += 32 * nw) {
+        const int quad = dK.q(e), kap = e - quad * K, col = quad << 2;
+        const int beta = (i == 0 || kap < rsplit) ? 0 : 1;
+        const int c1 = imin(col + 1, ncol - 1) - col, c2 = imin(col + 2, ncol - 1) - col,
+                  c3 = imin(col + 3, ncol - 1) - col;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (int al = 0; al < pam; ++al) {
+            PC crow = C + (al * Dl) * ldC + kap;
+            PC arow = A + col;
+            float x[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+            for (int l = 0; l < Dl; ++l, crow += ldC, arow += ncolA) {
+                const float cv = *crow;
+                x[0] = fmaf(cv, arow[0], x[0]);
+                x[1] = fmaf(cv, arow[c1], x[1]);
+                x[2] = fmaf(cv, arow[c2], x[2]);
+                x[3] = fmaf(cv, arow[c3], x[3]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                float w = 1.f;
+                if (i > 0) {
+                    const int ab = (col + u >= Dr ? 1 : 0) ^ beta, ub = al ^ bp;
+                    w = par == 0 ? wq[ub + 2 * ab] : wq[ab + 2 * ub];
+                }
+                acc[u] = fmaf(w, x[u], acc[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (col + u < ncol) {
+                M[(col + u) * csM + kap * rsM] = acc[u];
+                mx = fmaxf(mx, fabsf(acc[u]));
+            }
+    }
+    return mx;
+}
+template <int T>
+__device__ __noinline__ float mpo_apply_team(const Job* a, int w, int nw) {
+    return a->chip ? mpo_apply<Sh, Sh>(*a, shared_of(a->C), shared_of(a->A), shared_of(a->M), w, nw)
+                   : mpo_apply<float*, const float*>(*a, a->C, a->A, a->M, w, nw);
+}
+
+__device__ __forceinline__ void scale_floats(float* M, int n, float f, int first, int step) {
+    int e = first;
+#pragma unroll 1
+    for (; e + 3 * step < n; e += 4 * step) {
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = M[e + u * step];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) M[e + u * step] = x[u] * f;
+    }
+#pragma unroll 1
+    for (; e < n; e += step) M[e] *= f;
+}
+
+// Warp w's side of a team until the team's unit queue is empty.
+template <int T>
+__device__ __forceinline__ void serve(Job& job, int w) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (;;) {
+        team_barrier<T>();
+        const int kind = job.kind;
+        if (kind == kQuit) return;
+        if (kind == kApply) {
+            const float mx = warp_max(mpo_apply_team<T>(&job, w, T));
+            if (lane == 0) job.part[w] = mx;
+        } else if (kind == kNorms) {
+            if (job.chip) column_norms(shared_of(job.M), job.K, 1, job.cs, job.N, job.nrm, w, T);
+            else column_norms(job.M, job.K, job.rs, job.cs, job.N, job.nrm, w, T);
+        } else if (kind == kUpdate) {
+            if (job.chip)
+                reflect_columns_team<T, Sh>(shared_of(job.M), job.K, 1, job.cs, job.N, job.nrm, job.j, job.f, w, T);
+            else
+                reflect_columns_team<T, float*>(job.M, job.K, job.rs, job.cs, job.N, job.nrm, job.j, job.f, w, T);
+        } else if (kind == kApplyQ) {
+            apply_q_at<T>(job.chip, job.V0, job.tau0, job.nr0, job.V1, job.tau1, job.nr1, job.split, job.vrs, job.vcs,
+                          job.K, job.M, job.rs, job.cs, job.N, w, T);
+        } else {
+            scale_floats(job.M, job.N, job.f, 32 * w + lane, 32 * T);
+        }
+        team_barrier<T>();
+    }
+}
+
 // Plane rotation of every G-th row (stride gs) of two columns.
-__device__ __forceinline__ void rotate_columns(float* xp, float* xq, int rows, int gs, float cs, float sn) {
+template <class P>
+__device__ __forceinline__ void rotate_columns(P xp, P xq, int rows, int gs, float cs, float sn) {
 #pragma unroll 1
     for (; rows >= kAhead; rows -= kAhead) {
         float va[kAhead], vb[kAhead];
@@ -432,9 +693,10 @@ __device__ __forceinline__ void rotate_columns(float* xp, float* xq, int rows, i
 // FP32. Returns false when kMaxSweeps sweeps did not settle. (The entries of
 // X lie in one block of L n floats, those of W in one of n n: both layouts
 // are dense.)
-__device__ __forceinline__ bool jacobi(float* X, int L, int xrs, int xcs, int n, float* W, int wrs, int wcs,
-                                       unsigned long long* fl) {
-    const int lane = threadIdx.x & 31;
+template <class P>
+__device__ __forceinline__ bool jacobi(P X, int L, int xrs_, int xcs, int n, P W, int wrs_, int wcs,
+                                    unsigned long long* fl) {
+    const int lane = threadIdx.x & 31, xrs = kChip<P> ? 1 : xrs_, wrs = kChip<P> ? 1 : wrs_;
     float f2 = 0.f;
     const FDiv dL(L);
 #pragma unroll 1
@@ -477,7 +739,7 @@ __device__ __forceinline__ bool jacobi(float* X, int L, int xrs, int xcs, int n,
                 }
                 float al = 0.f, be = 0.f, ga = 0.f;
                 if (p >= 0) {
-                    const float *xp = X + p * xcs + g * xrs, *xq = X + q * xcs + g * xrs;
+                    P xp = X + p * xcs + g * xrs, xq = X + q * xcs + g * xrs;
                     int m = rows;
 #pragma unroll 1
                     for (; m >= kAhead; m -= kAhead) {
@@ -515,7 +777,7 @@ __device__ __forceinline__ bool jacobi(float* X, int L, int xrs, int xcs, int n,
                     const float cs = 1.f / sqrtf(fmaf(t, t, 1.f)), sn = cs * t;
 #pragma unroll 1
                     for (int h = 0; h < 2; ++h) {         // X, then W
-                        float* blk = h ? W + g * wrs : X + g * xrs;
+                        const P blk = h ? W + g * wrs : X + g * xrs;
                         const int cst = h ? wcs : xcs;
                         rotate_columns(blk + p * cst, blk + q * cst, h ? wrows : rows, h ? wgs : xgs, cs, sn);
                     }
@@ -536,6 +798,12 @@ __device__ __forceinline__ bool jacobi(float* X, int L, int xrs, int xcs, int n,
     if (lane == 0) *fl += 6ULL * L * ev + 6ULL * (L + n) * rt + 2ULL * L * n;
     __syncwarp();
     return ok;
+}
+
+template <class P>
+__device__ __noinline__ bool jacobi_call(P X, int L, int xrs, int xcs, int n, P W, int wrs, int wcs,
+                                         unsigned long long* fl) {
+    return jacobi<P>(X, L, xrs, xcs, n, W, wrs, wcs, fl);
 }
 
 // Per-unit state in shared memory beside the arena.
@@ -562,9 +830,11 @@ struct Placement {
 };
 
 // ---------------------------------------------------------------- the unit
+template <int T>
 struct Unit {
     const TruncArgs& a;
     Small& S;
+    Job* job;             // the team's (T > 1)
     float* arena;         // on-chip arena (a.arena floats)
     float* mps0;          // global MPS buffers (0 and 1)
     float* mps1;
@@ -603,8 +873,7 @@ struct Unit {
                 if (lane == 0) atomicAdd(a.bond_hist, 1ULL);   // bin 0: steps run in the spill arena
             } else { ovf = true; return false; }
             if (base != cbase) {
-#pragma unroll 1
-                for (int e = lane; e < csize; e += 32) base[e] = cptr[e];
+                copy_floats(base, cptr, csize, lane, 32);
             } else {                           // same arena, carry moved to its bottom
                 // (only when it sits at the top with room to spare below it)
 #pragma unroll 1
@@ -721,8 +990,7 @@ struct Unit {
             float* Co = out_ptr(P);
             // stage the old site (Dl x ncolA, row-major as stored)
             const float* Ag = src + S.Moff[sb][i];
-#pragma unroll 1
-            for (int e = lane; e < sA; e += 32) A[e] = Ag[e];
+            copy_floats(A, Ag, sA, lane, 32);
             __syncwarp();
             // on chip the rows of a column lie together (odd stride between
             // columns: lanes walking one column each hit distinct banks); in the
@@ -736,49 +1004,25 @@ struct Unit {
             bool any = false;
 #pragma unroll 1
             for (int bp = 0; bp < pb; ++bp) {
-                // M^{b'}[kappa][col] = sum_a w(a, a', beta(kappa), b') sum_l C[kappa][a Dl + l] A[l][col]
-                // (qubit (i-1, c); at i = d alpha_d is summed into the single column)
+                // (at i = d alpha_d is summed into the single column)
                 float mx = 0.f;
-                const int quads = (ncol + 3) >> 2;
+                const bool wide = T > 1 && K * ncol > 512;
                 if (i < d) {
-                    // four columns of one row at a time: one load of C for four
-                    // products, and four chains to overlap
-#pragma unroll 1
-                    for (int e = lane; e < K * quads; e += 32) {
-                        const int quad = dK.q(e), kap = e - quad * K, col = quad << 2;
-                        const int beta = (i == 0 || kap < rsplit) ? 0 : 1;
-                        const int c1 = imin(col + 1, ncol - 1) - col, c2 = imin(col + 2, ncol - 1) - col,
-                                  c3 = imin(col + 3, ncol - 1) - col;
-                        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-                        for (int al = 0; al < pam; ++al) {
-                            const float* crow = C + (al * Dl) * ldC + kap;
-                            const float* arow = A + col;
-                            float x[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-                            for (int l = 0; l < Dl; ++l, crow += ldC, arow += ncolA) {
-                                const float cv = *crow;
-                                x[0] = fmaf(cv, arow[0], x[0]);
-                                x[1] = fmaf(cv, arow[c1], x[1]);
-                                x[2] = fmaf(cv, arow[c2], x[2]);
-                                x[3] = fmaf(cv, arow[c3], x[3]);
-                            }
+                    Job m;
+                    m.kind = kApply;
+                    m.chip = P.base == arena;
+                    m.C = C; m.A = A; m.wq = wq; m.M = M; m.K = K; m.N = ncol; m.rs = rsM; m.cs = csM;
+                    m.ncolA = ncolA; m.Dl = Dl; m.Dr = Dr; m.ldC = ldC; m.pam = pam; m.par = par; m.bp = bp;
+                    m.i = i; m.rsplit = rsplit;
+                    if (wide) {
+                        if (lane == 0) *job = m;
+                        team_barrier<T>();
+                        mx = mpo_apply_team<T>(job, 0, T);
+                        team_barrier<T>();
 #pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                float w = 1.f;
-                                if (i > 0) {
-                                    const int ab = (col + u >= Dr ? 1 : 0) ^ beta, ub = al ^ bp;
-                                    w = par == 0 ? wq[ub + 2 * ab] : wq[ab + 2 * ub];
-                                }
-                                acc[u] = fmaf(w, x[u], acc[u]);
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (col + u < ncol) {
-                                M[(col + u) * csM + kap * rsM] = acc[u];
-                                mx = fmaxf(mx, fabsf(acc[u]));
-                            }
+                        for (int w = 1; w < T; ++w) mx = fmaxf(mx, job->part[w]);
+                    } else {
+                        mx = mpo_apply<float*, const float*>(m, C, A, M, 0, 1);
                     }
                 } else
 #pragma unroll 1
@@ -807,12 +1051,19 @@ struct Unit {
                 const int ex = exponent_of(mx);
                 if (ex > 126 || ex < -125) { bad = true; return; }
                 const float sc = pow2f(-ex);
-                __syncwarp();
-#pragma unroll 1
-                for (int e = lane; e < sM; e += 32) M[e] *= sc;
+                if (T > 1 && sM > 512) {
+                    if (lane == 0) { job->kind = kScale; job->M = M; job->N = sM; job->f = sc; }
+                    team_barrier<T>();
+                    scale_floats(M, sM, sc, lane, 32 * T);
+                    team_barrier<T>();
+                } else {
+                    __syncwarp();
+                    scale_floats(M, sM, sc, lane, 32);
+                }
                 __syncwarp();
                 // rank-revealing QR M^{b'} = Q [R; R22] P^T, R22 dropped
-                const int r = qrcp(M, K, rsM, csM, ncol, tau, piv, nrm, a.cutoff, rmax, &S.fl);
+                const int r = hot ? qrcp<T, ChipPtr<T>>(M, K, rsM, csM, ncol, tau, piv, nrm, a.cutoff, rmax, &S.fl, job)
+                                  : qrcp<T, float*>(M, K, rsM, csM, ncol, tau, piv, nrm, a.cutoff, rmax, &S.fl, job);
                 rb[bp] = r;
                 // reflectors (leading dimension K) and taus to the store
                 const int qsz = K * r + r;
@@ -889,8 +1140,9 @@ struct Unit {
             const bool chip = P.base == arena;
             const int small = 3 * N + 2 * mn;
             const int room = chip ? 0 : a.arena - small;
-            bool t_on = chip || sT <= room;
-            float* T = chip || !t_on ? P.work : arena;
+            const bool t_on = chip || sT <= room;
+            bool t_in = t_on;                     // (its reflectors, later)
+            float* Tm = chip || !t_on ? P.work : arena;
             float* X = P.work + sT;
             float* W = X + sX;
             float* tau = chip || room < 0 ? W + sW : arena + room;
@@ -906,26 +1158,27 @@ struct Unit {
                 const int n = dKi.q(e), kap = e - n * Ki;
                 const int bp = n >= Sr ? 1 : 0, s = n - bp * Sr;
                 const int rr = bp ? r1 : r0, off = bp ? r0 : 0;
-                T[n * csT + kap * rsT] = kap < rr ? G[s * ldG + off + kap] : 0.f;
+                Tm[n * csT + kap * rsT] = kap < rr ? G[s * ldG + off + kap] : 0.f;
             }
             __syncwarp();
             {
                 const float* Q0 = qst + S.Qoff[2 * i];
                 const float* Q1 = qst + S.Qoff[2 * i + 1];
-                apply_q(Q0, Q0 + Ki * r0, r0, Q1, Q1 + Ki * r1, r1, Sr, 1, Ki, Ki, T, rsT, csT, N, &S.fl);
+                apply_q_team<T>(t_on ? 1 : 0, Q0, Q0 + Ki * r0, r0, Q1, Q1 + Ki * r1, r1, Sr, 1, Ki, Ki, Tm, rsT, csT, N, &S.fl, job);
                 __syncwarp();
             }
             if (i == 0) {                         // Ki = 1: the orthogonality centre is the site
                 if (mo + N > a.caps.mps) { ovf = true; return; }
                 float* site = dst + mo;
 #pragma unroll 1
-                for (int e = lane; e < N; e += 32) site[e] = T[e * csT];
+                for (int e = lane; e < N; e += 32) site[e] = Tm[e * csT];
                 if (lane == 0) { S.Dnew[0] = 1; S.Moff[db][0] = mo; }
                 __syncwarp();
                 break;
             }
             // T P = Q_T [R; R22], R22 dropped; Jacobi on X = R^T (N x r')
-            const int rp = qrcp(T, Ki, rsT, csT, N, tau, piv, nrm, a.cutoff, mn, &S.fl);
+            const int rp = t_on ? qrcp<T, ChipPtr<T>>(Tm, Ki, rsT, csT, N, tau, piv, nrm, a.cutoff, mn, &S.fl, job)
+                                : qrcp<T, float*>(Tm, Ki, rsT, csT, N, tau, piv, nrm, a.cutoff, mn, &S.fl, job);
             if (rp == 0) { zero = true; return; }
             const int need = (N + rp) * rp;
             bool x_on = chip;
@@ -933,9 +1186,9 @@ struct Unit {
             if (!chip && need <= room) {
                 used = t_on && sT + need <= room ? sT : 0;
                 if (t_on && used == 0) {          // T (from here on its reflectors) makes way
-#pragma unroll 1
-                    for (int e = lane; e < sT; e += 32) P.work[e] = T[e];
-                    T = P.work;
+                    copy_floats(P.work, Tm, sT, lane, 32);
+                    Tm = P.work;
+                    t_in = false;
                     __syncwarp();
                 }
                 x_on = true;
@@ -948,10 +1201,16 @@ struct Unit {
 #pragma unroll 1
             for (int e = lane; e < rp * N; e += 32) {
                 const int j = dN.q(e), n = e - j * N;
-                X[n * rsX + j * csX] = j <= n ? T[n * csT + j * rsT] : 0.f;
+                X[n * rsX + j * csX] = j <= n ? Tm[n * csT + j * rsT] : 0.f;
             }
             __syncwarp();
-            if (!jacobi(X, N, rsX, csX, rp, W, rsW, csW, &S.fl)) timeout = true;
+            bool settled;
+            if constexpr (T > 1)
+                settled = x_on ? jacobi_call<Sh>(shared_of(X), N, 1, csX, rp, shared_of(W), 1, csW, &S.fl)
+                               : jacobi_call<float*>(X, N, rsX, csX, rp, W, rsW, csW, &S.fl);
+            else
+                settled = jacobi<float*>(X, N, rsX, csX, rp, W, rsW, csW, &S.fl);
+            if (!settled) timeout = true;
             // R = W Sigma U'^T: right vectors of T = P U', left = Q_T [W; 0];
             // keep k = min(chi, #{sigma > cutoff sigma_max}) largest
             float smax = 0.f;
@@ -1007,11 +1266,11 @@ struct Unit {
                 atomicAdd(a.bond_hist + (k < 64 ? k : 64), 1ULL);
             }
             __syncwarp();
-            apply_q(T, tau, rp, T, tau, rp, k, rsT, csT, Ki, Gn, 1, ldT, k, &S.fl);
+            apply_q_team<T>((chip || stage) ? (t_in ? 3 : rsT == 1 ? 1 : 0) : 0, Tm, tau, rp, Tm, tau, rp, k, rsT, csT, Ki,
+                            Gn, 1, ldT, k, &S.fl, job);
             __syncwarp();
             if (stage) {
-#pragma unroll 1
-                for (int e = lane; e < k * ldT; e += 32) Go[e] = Gn[e];
+                copy_floats(Go, Gn, k * ldT, lane, 32);
                 __syncwarp();
             }
             carry_is(P, Go, ldT * kcap, ldT);
@@ -1122,19 +1381,32 @@ struct Unit {
     }
 };
 
-// Shared memory of one unit: Small, then the arena (16-byte aligned).
-__host__ __device__ constexpr size_t small_bytes() { return (sizeof(Small) + 15) & ~size_t(15); }
+// Shared memory of one unit: Small, then the team's job (T > 1), then the
+// arena (16-byte aligned).
+template <int T>
+__host__ __device__ constexpr size_t small_bytes() {
+    return ((sizeof(Small) + 15) & ~size_t(15)) + (T > 1 ? (sizeof(Job) + 15) & ~size_t(15) : 0);
+}
+template <int T>
 __host__ __device__ constexpr size_t unit_bytes(int arena) {
-    return small_bytes() + (((size_t)arena * sizeof(float) + 15) & ~size_t(15));
+    return small_bytes<T>() + (((size_t)arena * sizeof(float) + 15) & ~size_t(15));
 }
 
+template <int T>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock, 4) trunc_kernel(TruncArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    unsigned char* mine = smem_raw + (size_t)warp * unit_bytes(a.arena);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, team = warp / T;
+    unsigned char* mine = smem_raw + (size_t)team * unit_bytes<T>(a.arena);
     Small& S = *reinterpret_cast<Small*>(mine);
-    float* arena = reinterpret_cast<float*>(mine + small_bytes());
-    const int64_t slot = (int64_t)blockIdx.x * kWarpsPerBlock + warp;
+    Job* job = T > 1 ? reinterpret_cast<Job*>(mine + ((sizeof(Small) + 15) & ~size_t(15))) : nullptr;
+    if constexpr (T > 1) {
+        if (warp % T) {
+            serve<T>(*job, warp % T);
+            return;
+        }
+    }
+    float* arena = reinterpret_cast<float*>(mine + small_bytes<T>());
+    const int64_t slot = (int64_t)blockIdx.x * (kWarpsPerBlock / T) + team;
     float* base = a.ws + slot * a.caps.slice();
     const unsigned long long units = a.in_list ? (unsigned long long)*a.in_count : 2ULL * (unsigned long long)a.B;
 #pragma unroll 1
@@ -1143,37 +1415,73 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, 4) trunc_kernel(TruncArgs
         if (lane == 0) idx = atomicAdd(a.next_unit, 1ULL);
         idx = __shfl_sync(kFull, idx, 0);
         if (idx >= units) break;
-        Unit u{a, S, arena, base, base + a.caps.mps, base + 2 * a.caps.mps,
-               base + 2 * a.caps.mps + a.caps.q};
+        Unit<T> u{a, S, job, arena, base, base + a.caps.mps, base + 2 * a.caps.mps,
+                  base + 2 * a.caps.mps + a.caps.q};
         u.run(a.in_list ? a.in_list[idx] : (int64_t)idx);
+    }
+    if constexpr (T > 1) {
+        if (lane == 0) job->kind = kQuit;
+        team_barrier<T>();
     }
 }
 
-}  // namespace trunc
+// Warps of a unit's team: the SM's sixteen, shared by the units its arenas
+// leave room for.
+constexpr int team_of(int arena) { return arena >= kTruncArenas[2] ? 4 : (arena >= kTruncArenas[1] ? 2 : 1); }
 
-int trunc_units_per_block() { return trunc::kWarpsPerBlock; }
-
-size_t trunc_smem_bytes(int arena) { return trunc::kWarpsPerBlock * trunc::unit_bytes(arena); }
-
-// (The attribute is set to the largest arena's size by every caller, so that
-// threads launching with different arenas do not undo each other's.)
-static bool allow_arenas() {
-    return cudaFuncSetAttribute(trunc::trunc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)trunc_smem_bytes(kTruncArenas[2])) == cudaSuccess;
+template <int T>
+bool allow() {
+    // (the largest arena of the team size, so that threads launching with
+    // different arenas do not undo each other's)
+    return cudaFuncSetAttribute(trunc_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(kWarpsPerBlock / T * unit_bytes<T>(kTruncArenas[T / 2]))) == cudaSuccess;
 }
-
-int trunc_blocks_per_sm(int arena) {
-    if (!allow_arenas()) return 0;
+template <int T>
+int resident(size_t bytes) {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, trunc::trunc_kernel, 32 * trunc::kWarpsPerBlock,
-                                                      trunc_smem_bytes(arena)) != cudaSuccess)
+    if (!allow<T>() || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, trunc_kernel<T>, 32 * kWarpsPerBlock,
+                                                                     bytes) != cudaSuccess)
         return 0;
     return n;
 }
 
+}  // namespace trunc
+
+int trunc_units_per_block(int arena) { return trunc::kWarpsPerBlock / trunc::team_of(arena); }
+
+size_t trunc_smem_bytes(int arena) {
+    switch (trunc::team_of(arena)) {
+        case 4: return trunc::unit_bytes<4>(arena);
+        case 2: return 2 * trunc::unit_bytes<2>(arena);
+    }
+    return 4 * trunc::unit_bytes<1>(arena);
+}
+
+int trunc_blocks_per_sm(int arena) {
+    const size_t bytes = trunc_smem_bytes(arena);
+    switch (trunc::team_of(arena)) {
+        case 4: return trunc::resident<4>(bytes);
+        case 2: return trunc::resident<2>(bytes);
+    }
+    return trunc::resident<1>(bytes);
+}
+
 bool launch_trunc(const TruncArgs& a, int blocks, cudaStream_t s) {
-    if (!allow_arenas()) return false;
-    trunc::trunc_kernel<<<blocks, 32 * trunc::kWarpsPerBlock, trunc_smem_bytes(a.arena), s>>>(a);
+    const size_t bytes = trunc_smem_bytes(a.arena);
+    const int threads = 32 * trunc::kWarpsPerBlock;
+    switch (trunc::team_of(a.arena)) {
+        case 4:
+            if (!trunc::allow<4>()) return false;
+            trunc::trunc_kernel<4><<<blocks, threads, bytes, s>>>(a);
+            break;
+        case 2:
+            if (!trunc::allow<2>()) return false;
+            trunc::trunc_kernel<2><<<blocks, threads, bytes, s>>>(a);
+            break;
+        default:
+            if (!trunc::allow<1>()) return false;
+            trunc::trunc_kernel<1><<<blocks, threads, bytes, s>>>(a);
+    }
     return cudaGetLastError() == cudaSuccess;
 }
 

@@ -1,4 +1,4 @@
-// Launcher of the rank-adaptive truncated sweep (one warp per unit).
+// Launcher of the rank-adaptive truncated sweep.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -7,9 +7,9 @@
 namespace mld {
 
 // Capacities of one unit's shapes and global slice (floats). The first pass
-// over all units runs on every resident warp with the smallest that hold
-// chi (bond 48, 64 or 128: 2.25, 4.5 or 17.8 MB per warp); units that exceed
-// them are decoded by a second pass with the large ones on few warps.
+// over all units runs on every resident team with the smallest that hold
+// chi (bond 48, 64 or 128: 2.25, 4.5 or 17.8 MB per unit); units that exceed
+// them are decoded by a second pass with the large ones, a unit per SM.
 struct TruncCaps {
     int max_bond;        // kept bond per cut
     int max_rows;        // carry rows
@@ -22,12 +22,13 @@ constexpr TruncCaps kTruncSmall{48, 192, 128 * 1024, 256 * 1024, 64 * 1024};
 constexpr TruncCaps kTruncMid{64, 256, 256 * 1024, 512 * 1024, 128 * 1024};
 constexpr TruncCaps kTruncLarge{128, 512, 1024 * 1024, 2048 * 1024, 384 * 1024};
 
-// On-chip work arena of a unit (floats): 16, 8 or 4 warps share an SM. Batches
-// that leave an SM at most 8 or 4 units get the larger ones: their time is the
-// heaviest unit's, whose large steps then stay on chip (d = 25, chi = 64, 515
-// syndromes: 130 ms with 8 warps, 153 with 16; d = 17, p = 0.17, 128 syndromes:
-// 133 ms with 4, 149 with 8, 181 with 16; under load more warps are faster:
-// d = 17, 8,192 syndromes 237 ms with 16, 279 with 8, 450 with 4).
+// On-chip work arena of a unit (floats): 16, 8 or 4 units share an SM's sixteen
+// warps, in teams of 1, 2 or 4. Batches that leave an SM at most 8 or 4 units
+// get the larger ones: their time is the heaviest unit's, whose large steps
+// then stay on chip and are shared by its team (d = 25, chi = 64, 515 syndromes:
+// 114 ms with 8 units, 137 with 4; d = 17, p = 0.17, 128 syndromes: 100 ms with
+// 4, 149 with 8 and 181 with 16 single warps; under load more units are faster:
+// d = 17, 2,048 syndromes 91 ms with 16, 121 with 8).
 constexpr int kTruncArenas[3] = {3072, 6500, 13500};
 constexpr int trunc_arena(int64_t units, int sms) {
     return kTruncArenas[units <= 4 * (int64_t)sms ? 2 : (units <= 8 * (int64_t)sms ? 1 : 0)];
@@ -55,9 +56,9 @@ struct TruncArgs {
     unsigned long long* bond_hist;   // [65]: kept bonds k of every truncating cut (k >= 64 in the last bin)
 };
 
-// Units (warps) per block, dynamic shared memory per block for an arena of
+// Units per block, dynamic shared memory per block for an arena of
 // `arena` floats per unit, resident blocks per SM (0 on error), and the launch.
-int trunc_units_per_block();
+int trunc_units_per_block(int arena);
 size_t trunc_smem_bytes(int arena);
 int trunc_blocks_per_sm(int arena);
 bool launch_trunc(const TruncArgs& a, int blocks, cudaStream_t s);
