@@ -232,10 +232,10 @@ mld_status mld_autotune(const mld_code* code, int chi, int precision, int64_t sa
  *              treated as independent) is ADDED to it.
  * Each qubit factor's environment is contracted exactly, so chi must not
  * truncate (MLD_ERR_UNSUPPORTED otherwise) and d <= 13. The left and right
- * boundary states are kept dense (the right states are carried back through
- * each column by the transposed factors): on chip for d <= 11; at d = 13 the
- * states inside a column (128 KB each) live in a device workspace of about
- * 1.7 MB per resident block, the corner-column states on chip. The left
+ * boundary states are kept as their entries (the right states are carried
+ * back through each column by the transposed factors): in registers for
+ * d <= 11; at d = 13 the states inside a column (128 KB each) live in a device
+ * workspace of about 1.7 MB per resident block. The left
  * state at every column boundary is stored by the forward pass (a
  * checkpoint per column) and the states inside a column are recomputed from
  * it during the backward pass. FP32 contraction, FP64

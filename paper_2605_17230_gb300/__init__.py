@@ -282,7 +282,8 @@ class Code:
         return logP, am
 
     def decode_xz(self, px, pz, syndromes, precision=MLD_FP32, with_argmax=True, stream=None):
-        """Kac-Ward decode under independent X/Z noise: px, pz float32 [n]
+        """Exact decode under independent X/Z noise (MLD_FP32: Kac-Ward
+        determinants; MLD_FP64: column transfer): px, pz float32 [n]
         CUDA tensors (pz None: bit-flip noise). Returns (logP float64 [B][4],
         argmax uint8 [B] or None)."""
         import torch
@@ -422,7 +423,7 @@ def mld_decode_dem(code, mech_qubit, mech_pauli, mech_p, syndromes, B, logP, arg
 
 
 def mld_decode_xz(code, px, pz, syndromes, B, precision, logP, argmax=None, stream=None):
-    """C-ABI mld_decode_xz (Kac-Ward, independent X/Z noise): px, pz (or None
+    """C-ABI mld_decode_xz (exact, independent X/Z noise): px, pz (or None
     for bit-flip noise), syndromes and outputs are torch CUDA tensors."""
     _check(load().mld_decode_xz(code, _ptr(px), _ptr(pz), _ptr(syndromes), int(B), int(precision),
                                 _ptr(logP), _ptr(argmax), _stream(stream)), "mld_decode_xz")

@@ -1,5 +1,5 @@
-// Steps of the dense column transfer shared by the untruncated kernels that
-// keep the boundary state dense (the adjoint and the d = 13 forward sweep).
+// Steps of the dense column transfer of the d = 13 adjoint, which keeps the
+// boundary state dense.
 //
 // Within column c the state before factor r (qubit (r, c)) is indexed by d+2
 // bits: bits 0..r hold beta_0..beta_r (corner column c+1), bits r+1..d hold

@@ -1,4 +1,6 @@
-// Dense adjoint of the untruncated sweep, d = 3..13: d ln Z_l / d p_{q,P}.
+// Dense adjoint of the untruncated sweep at d = 13: d ln Z_l / d p_{q,P}
+// (mld_grad_gate.cu runs d = 3..11; its states and adjoint states in
+// registers would be 2 x 128 of them a lane here).
 // (Each block sums its units' gradients in a fixed order and a second
 // kernel adds the blocks' sums in block order: reruns are bit-identical.)
 //
@@ -7,16 +9,15 @@
 // probabilities, which the estimation of Eq. 10 back-propagates). The exact
 // boundary state over one corner column has at most 2^(d+1) entries (one
 // plaquette variable per row, absent plaquettes pinned to 0), so the states
-// are kept dense: on chip for d <= 11; at d = 13 (128 KB per state inside a
-// column) the states inside a column live in the block's global slice and
-// only the two corner-column states R stay on chip. One thread block owns one
-// (syndrome, class) unit:
+// are kept dense: 128 KB per state inside a column, so these live in the
+// block's global slice and only the two corner-column states R stay on chip.
+// One thread block owns one (syndrome, class) unit:
 //   forward   L_{c+1} = T_c L_c for c = 0..d-1, T_c applied qubit factor by
 //             qubit factor to states over d+2 bits and rescaled by a power of
 //             two per column; L_1..L_{d-1} go to the block's global slice, and
 //             ln Z_l = ln sum L_d + the accumulated exponents.
 //   backward  for c = d-1..0: the transposed factors carry R_{c+1} back
-//             through column c (the states G_r kept in shared memory) and G_0
+//             through column c (the states G_r kept in the slice) and G_0
 //             gives R_c; then the factors are re-applied from L_c, and each
 //             factor's environment is the contraction of the state before it
 //             with G after it, bucketed by the factor's weight slot.
@@ -48,42 +49,27 @@ using namespace dense;
 
 template <int D>
 struct GradShape {
-    static_assert(D % 2 == 1, "odd distances only");
+    static_assert(D == 13, "smaller distances: mld_grad_gate.cu");
     static constexpr int N = D * D;
     static constexpr int HALF = 1 << (D + 1);       // states over one corner column
     static constexpr int SIZE = HALF << 1;          // states inside a column (one more bit)
     static constexpr int REST1 = SIZE >> 3;         // rests of a single step (eight entries each)
     static constexpr int REST2 = SIZE >> 4;         // rests of a pair step (sixteen entries each)
-    static constexpr int NT = REST2 >= 512 ? 512 : (REST2 >= 128 ? 128 : 32);
-    // d >= 11: one block fills an SM's shared memory, so L_c is read from the
-    // block's global slice, each step's environment sums are reduced at once,
-    // and the representative's bits are recomputed where they are needed
-    static constexpr bool BIG = D >= 11;
-    // d >= 13: the G states (the states inside a column) are in the block's
-    // global slice too; a thread takes several rests per step
-    static constexpr bool HUGE = D >= 13;
+    static constexpr int NT = 512;                  // four rests of a pair step a thread
     static constexpr int NW = NT / 32;
     static constexpr int NG = (D + 1) / 2;          // stored G states: r = 0, 2, .., d-1
     // shared memory (floats)
-    static constexpr int off_w = 0;                          // 4N factor weights (slot order Wp)
-    static constexpr int off_g = (4 * N + 3) & ~3;           // NG states of SIZE (on chip unless HUGE)
-    static constexpr int off_l = off_g + (HUGE ? 0 : NG * SIZE);   // HALF: L_c for the environment pass
-    static constexpr int off_ra = off_l + (BIG ? 0 : HALF);   // HALF: R_{c+1} (and staging)
+    static constexpr int off_w = 0;                           // 4N factor weights (slot order Wp)
+    static constexpr int off_ra = (4 * N + 3) & ~3;           // HALF: R_{c+1} (and staging)
     static constexpr int off_rb = off_ra + HALF;              // HALF: R_c being formed
-    static constexpr int off_red = off_rb + HALF;             // per-warp environment sums:
-    static constexpr int RED = BIG ? NW * 8 : D * NW * 4;     //   of one step (BIG) or of the column
-    static constexpr int off_env = off_red + RED;             // D x 4 environments of a column
+    static constexpr int off_red = off_rb + HALF;             // per-warp environment sums of one step
+    static constexpr int off_env = off_red + NW * 8;          // D x 4 environments of a column
     static constexpr int off_misc = off_env + D * 4;          // 32: per-warp reductions
-    static constexpr int off_rep = off_misc + 32;             // N ints: representative x + 2z
-    static constexpr int floats = off_rep + (BIG ? 0 : N);
+    static constexpr int floats = off_misc + 32;
     static constexpr int lfloats = (D - 1) * HALF;            // global: L_1..L_{d-1}
-    static constexpr int goff = lfloats + 8 * N;               // + the block's 4N double gradient sums
-    static constexpr int slice = goff + (HUGE ? NG * SIZE : 0);   // + the G states (HUGE)
+    static constexpr int goff = lfloats + 8 * N;              // + the block's 4N double gradient sums
+    static constexpr int slice = goff + NG * SIZE;            // + the G states (before even factors)
     static_assert(goff % 4 == 0 && slice % 4 == 0, "16-byte aligned slices");
-    // blocks per SM that shared memory allows (the register budget is held to it)
-    static constexpr int FIT0 = (227 * 1024) / (floats * 4 + 1024);
-    static constexpr int FIT = FIT0 < 1 ? 1 : FIT0;   // one block of up to 227 KB always fits
-    static constexpr int MINB = FIT < 16 ? FIT : 16;
     static_assert(floats * 4 <= 227 * 1024, "a block's shared memory is at most 227 KB");
 };
 
@@ -92,7 +78,7 @@ template <int D>
 __device__ __forceinline__ constexpr int gslot(int r) { return r == D ? (D + 1) / 2 : r / 2; }
 
 // Shared-memory position of entry e of a stored state with layout index lay
-// (the state before factor lay; d >= 7). The 32 lanes of a warp own 32
+// (the state before factor lay). The 32 lanes of a warp own 32
 // consecutive rests, i.e. vary the five lowest index bits that the step
 // leaves fixed; when the step touches bank bits (0..4), a plain layout puts
 // the warp on 4 to 16 banks. XORing bits 5, 6 and 7 into the bank bits with
@@ -106,7 +92,6 @@ __device__ __forceinline__ constexpr int swz_mask(int lay, int bit) {
 }
 template <int D>
 __device__ __forceinline__ int phys(int e, int lay) {
-    if (D < 7) return e;
     return e ^ (((e >> 5) & 1) ? swz_mask(lay, 5) : 0) ^ (((e >> 6) & 1) ? swz_mask(lay, 6) : 0) ^
            (((e >> 7) & 1) ? swz_mask(lay, 7) : 0);
 }
@@ -232,21 +217,19 @@ __device__ __forceinline__ float reduce_scatter4(float (&v)[4], int lane) {
 }
 
 template <int D>
-__global__ void __launch_bounds__(GradShape<D>::NT, GradShape<D>::MINB) grad_dense_kernel(GradDenseArgs g) {
+__global__ void __launch_bounds__(GradShape<D>::NT, 1) grad_dense_kernel(GradDenseArgs g) {
     using S = GradShape<D>;
     constexpr int N = S::N, HALF = S::HALF, SIZE = S::SIZE, NT = S::NT, NW = S::NW;
     extern __shared__ float4 smem4[];
     float* sm = reinterpret_cast<float*>(smem4);
     float* wts = sm + S::off_w;
     float* Lg = g.lws + (size_t)blockIdx.x * S::slice;
-    float* G = S::HUGE ? Lg + S::goff : sm + S::off_g;   // G + gslot(r) * SIZE: the state before factor r
-    float* Lb = sm + S::off_l;             // (d <= 9 only)
+    float* G = Lg + S::goff;   // G + gslot(r) * SIZE: the state before factor r
     float* Rcur = sm + S::off_ra;
     float* Rnxt = sm + S::off_rb;
     float* red = sm + S::off_red;
     float* env = sm + S::off_env;
     float* misc = sm + S::off_misc;
-    int* rep = reinterpret_cast<int*>(sm + S::off_rep);   // (d <= 9 only)
     double* acc = reinterpret_cast<double*>(Lg + S::lfloats);   // this block's dL/dp, summed in unit order
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -278,7 +261,6 @@ __global__ void __launch_bounds__(GradShape<D>::NT, GradShape<D>::MINB) grad_den
                 const int xx = x ^ (uv & 1), zz = z ^ (uv >> 1);
                 wts[4 * q + j] = row[xx ? (zz ? 2 : 1) : (zz ? 3 : 0)];
             }
-            if constexpr (!S::BIG) rep[q] = x + 2 * z;
         }
         {
             const int pm0 = present_rows<D>(0);
@@ -357,11 +339,6 @@ __global__ void __launch_bounds__(GradShape<D>::NT, GradShape<D>::MINB) grad_den
             for (int bi = tid; bi < HALF; bi += NT) Rcur[bi] = (bi & ~pmd) == 0 ? 1.f : 0.f;   // R_d
         }
         for (int c = D - 1; c >= 0; --c) {
-            if constexpr (!S::BIG) {
-                const int pm0 = present_rows<D>(0);
-                for (int bi = tid; bi < HALF; bi += NT)
-                    Lb[bi] = c == 0 ? ((bi & ~pm0) == 0 ? 1.f : 0.f) : Lg[(c - 1) * HALF + bi];
-            }
             __syncthreads();
             {
                 float W[4];
@@ -431,10 +408,7 @@ __global__ void __launch_bounds__(GradShape<D>::NT, GradShape<D>::MINB) grad_den
                         for (int m = 0; m < 16; ++m) {
                             const int lg = core | (m & 7) | ((m >> 3) << (D + 1));
                             const int li = left_index<D>(lg);
-                            if constexpr (S::BIG)
-                                X[m] = c == 0 ? ((li & ~present_rows<D>(0)) == 0 ? 1.f : 0.f) : Lg[(c - 1) * HALF + li];
-                            else
-                                X[m] = Lb[li];
+                            X[m] = c == 0 ? ((li & ~present_rows<D>(0)) == 0 ? 1.f : 0.f) : Lg[(c - 1) * HALF + li];
                             Gz[m] = Gn[o2[m]];
                         }
                     } else {
@@ -466,45 +440,27 @@ __global__ void __launch_bounds__(GradShape<D>::NT, GradShape<D>::MINB) grad_den
                     for (int m = 0; m < 16; ++m) Fb[o2[m]] = Z[m];
                 });
                 const float tot = reduce_scatter8(e, lane);
-                if ((lane & 3) == 0) {
-                    const int slot = lane >> 2;
-                    if constexpr (S::BIG) red[warp * 8 + slot] = tot;
-                    else red[((r + (slot >> 2)) * NW + warp) * 4 + (slot & 3)] = tot;
+                if ((lane & 3) == 0) red[warp * 8 + (lane >> 2)] = tot;
+                __syncthreads();
+                if (tid < 8) {
+                    float sum = 0.f;
+                    for (int w = 0; w < NW; ++w) sum += red[w * 8 + tid];
+                    env[(r + (tid >> 2)) * 4 + (tid & 3)] = sum;
                 }
                 __syncthreads();
-                if constexpr (S::BIG) {
-                    if (tid < 8) {
-                        float sum = 0.f;
-                        for (int w = 0; w < NW; ++w) sum += red[w * 8 + tid];
-                        env[(r + (tid >> 2)) * 4 + (tid & 3)] = sum;
-                    }
-                    __syncthreads();
-                }
                 Fa = Fb;
             }
             {
                 float e[4] = {0.f, 0.f, 0.f, 0.f};
                 for (int rs = tid; rs < S::REST1; rs += NT) single_environment<D, true>(Fa, Rcur, D - 1, rs, e);
                 const float tot = reduce_scatter4(e, lane);
-                if ((lane & 7) == 0) {
-                    if constexpr (S::BIG) red[warp * 8 + (lane >> 3)] = tot;
-                    else red[((D - 1) * NW + warp) * 4 + (lane >> 3)] = tot;
-                }
+                if ((lane & 7) == 0) red[warp * 8 + (lane >> 3)] = tot;
                 __syncthreads();
             }
-            if constexpr (S::BIG) {
-                if (tid < 4) {
-                    float sum = 0.f;
-                    for (int w = 0; w < NW; ++w) sum += red[w * 8 + tid];
-                    env[(D - 1) * 4 + tid] = sum;
-                }
-            } else {
-                for (int t = tid; t < D * 4; t += NT) {
-                    float s = 0.f;
-#pragma unroll
-                    for (int w = 0; w < NW; ++w) s += red[((t >> 2) * NW + w) * 4 + (t & 3)];
-                    env[t] = s;
-                }
+            if (tid < 4) {
+                float sum = 0.f;
+                for (int w = 0; w < NW; ++w) sum += red[w * 8 + tid];
+                env[(D - 1) * 4 + tid] = sum;
             }
             __syncthreads();
             // dZ/dp_{q,P} = env / <R|T|L>, with <R|T|L> = sum_j env_j Wp_j of factor 0
@@ -519,21 +475,15 @@ __global__ void __launch_bounds__(GradShape<D>::NT, GradShape<D>::MINB) grad_den
                 const float eu = env[4 * r + (par ? ((uv & 1) << 1) | (uv >> 1) : uv)];
                 if (zc > 0.f) {
                     const int q = r * D + c;
-                    int rx, rz;
-                    if constexpr (S::BIG) {
-                        rx = 0; rz = 0;
-                        const uint64_t* mk = g.dmask + (size_t)q * 2 * g.words;
-                        for (int w = 0; w < g.words; ++w) {
-                            const uint64_t sw = g.syn[b * g.words + w];
-                            rx ^= __popcll(sw & mk[w]) & 1;
-                            rz ^= __popcll(sw & mk[g.words + w]) & 1;
-                        }
-                        if ((cls & 1) && c == 0) rx ^= 1;
-                        if ((cls & 2) && r == 0) rz ^= 1;
-                    } else {
-                        rx = rep[q] & 1;
-                        rz = rep[q] >> 1;
+                    int rx = 0, rz = 0;
+                    const uint64_t* mk = g.dmask + (size_t)q * 2 * g.words;
+                    for (int w = 0; w < g.words; ++w) {
+                        const uint64_t sw = g.syn[b * g.words + w];
+                        rx ^= __popcll(sw & mk[w]) & 1;
+                        rz ^= __popcll(sw & mk[g.words + w]) & 1;
                     }
+                    if ((cls & 1) && c == 0) rx ^= 1;
+                    if ((cls & 2) && r == 0) rz ^= 1;
                     const int xx = rx ^ (uv & 1), zz = rz ^ (uv >> 1);
                     acc[4 * q + (xx ? (zz ? 2 : 1) : (zz ? 3 : 0))] += up * (double)(eu / zc);
                 }

@@ -18,7 +18,7 @@
 // their midpoint, I - Lambda is banded (bandwidth about 3d) apart from the tie
 // path's middle edge, which is ordered last as a two-row, two-column border,
 // and the sector edge's two columns are the last two of the band. One warp
-// (d <= 15) or one block of four warps (above, with look-ahead: while warps 2
+// (d <= 13) or one block of four warps (above, with look-ahead: while warps 2
 // and 3 apply step k to columns k+2.., warp 0 applies it to column k+1 and
 // takes step k+1's pivot and multipliers, and warp 1 writes the entering row)
 // eliminates one matrix with partial pivoting, streaming: only the rows and

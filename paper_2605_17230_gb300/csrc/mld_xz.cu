@@ -3,10 +3,9 @@
 // each part's coset sum is a planar random-bond Ising partition function.
 // Swept column by column its boundary state is one bit per plaquette of the
 // part's type, h = (d-1)/2 bits: 256 entries at d = 17, 4,096 at d = 25. Every
-// term is a product of probabilities, so nothing cancels: FP32 keeps FP32
-// relative accuracy at any rate, where a Kac-Ward determinant (a signed sum)
-// loses ln Z at low rates. For h <= 12 the transfer is also the smaller
-// computation: 0.5 MFLOP a syndrome at d = 17 against 6.0 executed by a banded
+// term is a product of probabilities, so nothing cancels at any rate, where a
+// Kac-Ward determinant (a signed sum) loses ln Z at low rates. For h <= 12 the
+// transfer is also the smaller computation: 0.5 MFLOP a syndrome at d = 17 against 6.0 executed by a banded
 // elimination of the 2|E| x 2|E| matrix, without its chain of pivots.
 //
 // The z part: Z-type plaquettes, at the odd row positions of a corner column.
@@ -233,8 +232,7 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
         } else {
             // One gate body (1,300 instructions) for all row pairs: unrolled
             // over the twelve of d = 25 it is 230 KB of code and fetching it
-            // takes five times the arithmetic (8.3 ms against 1.9 for 1,024
-            // syndromes).
+            // takes as long again (8.3 ms against 4.2 for 1,024 syndromes).
             unsigned char* X = xch + (size_t)unit * S::REGION * S::VB;
 #pragma unroll 1
             for (int c = 0; c < D; ++c) {

@@ -1,6 +1,6 @@
 """Chunked decoding of a syndrome array larger than one launch, with resume
-(the boundary-MPS decode, ``decode_to_files``, and the Kac-Ward decode under
-independent X/Z noise, ``decode_xz_to_files``).
+(``decode_to_files``, and the decode under independent X/Z noise,
+``decode_xz_to_files``).
 
 Decoding is stateless per syndrome, so a long job is a sequence of chunks. The
 results go to two ``.npy`` files opened as memory maps (``<prefix>.logp.npy``,
@@ -128,7 +128,7 @@ def decode_to_files(code, noise, syndromes: np.ndarray, chi: int, prefix: str, c
 
 def decode_xz_to_files(code, px, pz, syndromes: np.ndarray, prefix: str, chunk: int = 1 << 18,
                        precision: int = MLD_FP32, resume: bool = True, on_chunk=None):
-    """The same for the Kac-Ward decode under independent X/Z noise
+    """The same for the decode under independent X/Z noise
     (``mld_decode_xz``): px, pz are CUDA float32 tensors [n] (pz None for
     bit-flip noise). The progress record also holds the method and a
     fingerprint of the rates, so a job resumed with other rates is refused."""
