@@ -44,13 +44,10 @@ TF32_PER_BF16 = 1.1 / 2.25          # nominal dense TF32 / BF16 tensor rates of 
 # DRAM bytes per syndrome of the decode kernel (dram__bytes_read.sum + write.sum of one ncu
 # capture of 8,192 syndromes of the headline kernel), valid only for the kernel sources they
 # were taken on: any change to them makes the traffic unknown (null).
-TRAFFIC_SOURCES_SHA = "a2b856029856e7f9"
-TRAFFIC_BYTES_PER_SYNDROME = {0: (286.208e3 + 1.536e3) / 8192, 2: (286.208e3 + 0.0) / 8192}
-
-
-# sources of the headline kernel (decode_exact_kernel<9, *>): its plan, layout and templates (the
-# host-side code object declared beside them in mld_internal.h does not enter the kernel)
-TRAFFIC_SOURCES = ("mld_plan.h", "mld_exact_impl.cuh", "mld_exact.h", "mld_exact.cu")
+TRAFFIC_SOURCES_SHA = "b992a96b56cd3cbb"
+TRAFFIC_BYTES_PER_SYNDROME = {0: 187.328e3 / 8192, 2: 187.328e3 / 8192}
+# sources of the headline kernel (gate_decode_kernel<9, *>)
+TRAFFIC_SOURCES = ("mld_gate.cuh", "mld_gate.h", "mld_gate.cu")
 
 
 def kernel_sources_sha():
@@ -219,14 +216,8 @@ MIXED_CHI = {3: 16, 5: 16, 7: 16, 9: 32, 11: 32, 13: 64}
 
 # what a mixed-precision request runs at each d of the mixed batch
 PRODUCT_PATH = {
-    0: "FP32 FFMA products (the split-TF32 path is slower at this d; a mixed request runs the FP32 kernel)",
-    9: "split-TF32 mma.sync tensor-core products (hi.hi + hi.lo + lo.hi) for data-site products of at "
-       "least 32x16x32, FP32 elsewhere",
-    11: "dense-state FP32 column transfer (untruncated chi; the faster exact kernel at this d, 2.6M "
-        "against 2.1M syndromes/s for the split-TF32 boundary-MPS kernel; a mixed request runs the same "
-        "kernel)",
-    13: "dense-state FP32 column transfer (untruncated chi; no product is MMA-shaped; a mixed request "
-        "runs the same kernel)",
+    0: "FP32 column transfer, one 2x2 gate per qubit (untruncated chi; no product is MMA-shaped; a mixed request "
+       "runs the same kernel)",
 }
 
 
@@ -872,9 +863,9 @@ def main():
                          "ler: logical-error rates of the d/p grid against the oracle; point: one (d, chi, p) "
                          "decode point, FP32 and mixed; kw: the Kac-Ward decode under independent X/Z "
                          "noise against the boundary-MPS decode of the same syndromes; kw-threshold: "
-                         "logical-error rates under bit-flip noise around the 10.9% threshold, exact; kw-chi: "
+                         "logical-error rates under bit-flip noise around the 10.9%% threshold, exact; kw-chi: "
                          "truncated boundary-MPS decisions against exact MLD at d=17, 25; threshold: "
-                         "logical-error rates under depolarizing noise around the 18.9% threshold")
+                         "logical-error rates under depolarizing noise around the 18.9%% threshold")
     ap.add_argument("--kw-d", type=int, nargs="+", default=[9, 13, 17, 25], help="kw: distances")
     ap.add_argument("--kw-p", type=float, default=0.10, help="kw: X and Z flip rate per qubit")
     ap.add_argument("--kw-batch", type=int, default=0, help="kw: syndromes per decode (0: by d)")
@@ -901,7 +892,7 @@ def main():
     ap.add_argument("--point-p", type=float, default=0.10, help="point: depolarizing p")
     ap.add_argument("--point-batch", type=int, default=32768, help="point: syndromes per decode")
     ap.add_argument("--point-exact-kernel", type=int, default=0, choices=[0, 1, 2],
-                    help="point, untruncated chi: 0 by d, 1 boundary-MPS kernel, 2 dense-state kernel")
+                    help="point, untruncated chi: 0 the column transfer, 1 boundary-MPS kernel, 2 as 0")
     ap.add_argument("--mixed-total", type=int, default=1 << 20)
     args = ap.parse_args()
     rank, world = _env_int("RANK", 0), _env_int("WORLD_SIZE", 1)
@@ -1023,8 +1014,8 @@ def main():
     e2e_val = world * Bn * e2e_steps / e2e_dt
 
     # roofline of the dominant kernel (the fused decode kernel): counted flops
-    # of the executed schedule / its CUDA-event time (the argmax kernel is
-    # < 1% of the step and is included in the timing), against the FP32 FMA
+    # of the executed schedule / its CUDA-event time (the pass over tied
+    # syndromes, a tenth of the step, is included), against the FP32 FMA
     # rate measured on this GPU by an FFMA microbenchmark (outside the timed
     # region); the tensor fraction sets the same flops against the dense TF32
     # rate (the measured BF16 cuBLAS peak scaled by the nominal TF32/BF16 ratio)
@@ -1040,12 +1031,12 @@ def main():
         "metric": METRIC, "value": value, "unit": "syndromes/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": 1e3 * t_max / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None,
-        "dtype": "tf32x3+f32" if prec_mixed == mld.MLD_MIXED_TF32 else "f32", "data": "synthetic",
+        "dtype": "f32", "data": "synthetic",
         "config": {"workload": f"rotated d={D}, depolarizing p={P}, chi={CHI}, {Bn} syndromes per GPU per step, "
                                f"4 cosets + argmax",
                    "global_batch": Bn * world, "l2": "flushed between timed steps (256 MiB write)",
-                   "precision": ("mixed: MPO.MPS data-site products on tensor cores from split TF32 operands "
-                                 "(hi.hi + hi.lo + lo.hi), FP32 accumulate; everything else FP32")
+                   "precision": ("mixed precision asked for; the column transfer that serves it at this chi "
+                                 "computes in FP32 (tied syndromes are decided by the split-TF32 sweep)")
                    if prec_mixed == mld.MLD_MIXED_TF32 else "fp32 (mixed path failed the 1e-3 bound)"},
         "fp32": {"value": value32, "ms_per_step": 1e3 * t32 / args.steps},
         "mixed_vs_fp32_max_abs_dlogP": dlogp,
