@@ -858,13 +858,21 @@ mld_status decode_truncated(mld_code* C, const mld::Plan& P, const mld::SiteStep
         if (cudaMalloc(&C->d_tctl, kTctlBytes) != cudaSuccess) return MLD_ERR_NOMEM;
         if (cudaMemset(C->d_tctl, 0, kTctlBytes) != cudaSuccess) return MLD_ERR_CUDA;
     }
-    if (2 * units > C->ovf_cap) {
+    // the two overflow lists, and the order of the syndromes where units queue:
+    // heaviest first (d = 17, chi = 32, 2,048 syndromes 91 -> 78 ms, 8,192 237 ->
+    // 208; d = 25, chi = 64, 1,500 231 -> 211; not where a quarter or less waits:
+    // 1,300 at d = 17 took 72 for 70, the heavy units slowing one another)
+    const bool queued = 4 * units > 5 * blocks1 * upb;
+    const int64_t lists = 2 * units + (queued ? B : 0);
+    if (lists > C->ovf_cap) {
         cudaFree(C->d_ovf);
         C->d_ovf = nullptr;
         C->ovf_cap = 0;
-        if (cudaMalloc(&C->d_ovf, (size_t)2 * units * sizeof(int64_t)) != cudaSuccess) return MLD_ERR_NOMEM;
-        C->ovf_cap = 2 * units;
+        if (cudaMalloc(&C->d_ovf, (size_t)lists * sizeof(int64_t)) != cudaSuccess) return MLD_ERR_NOMEM;
+        C->ovf_cap = lists;
     }
+    int64_t* by_weight = queued ? C->d_ovf + 2 * units : nullptr;
+    if (queued && !mld::launch_order(syn, B, C->words, by_weight, s)) return MLD_ERR_CUDA;
     char* ctl = static_cast<char*>(C->d_tctl);
     // queue heads and overflow counts start at zero (flops and histogram accumulate)
     if (cudaMemsetAsync(ctl, 0, 24, s) != cudaSuccess) return MLD_ERR_CUDA;
@@ -885,6 +893,7 @@ mld_status decode_truncated(mld_code* C, const mld::Plan& P, const mld::SiteStep
     ta.caps = caps1;
     ta.ws = C->d_tws;
     ta.next_unit = reinterpret_cast<unsigned long long*>(ctl);
+    ta.order = by_weight;
     ta.in_list = nullptr;
     ta.in_count = nullptr;
     ta.ovf_list = C->d_ovf;

@@ -51,8 +51,9 @@
 // not unrolled beyond loading four rows ahead of their stores, copies run
 // over flattened indices, arg-max and maximum are integer reductions, and
 // small batches get larger arenas and teams. Measured on GB300: d = 17,
-// chi = 32, 2,048 syndromes 91 ms (178 with loops unrolled by the compiler,
-// spilled steps walking global columns), 8,192 syndromes 237 ms (449); d = 25,
+// chi = 32, 2,048 syndromes 78 ms (91 with the units in the caller's order, 178
+// with loops unrolled by the compiler, spilled steps walking global columns),
+// 8,192 syndromes 208 ms (237, 449); d = 25,
 // chi = 64, 515 syndromes 114 ms (130 without teams; 321); d = 17, p = 0.17, 32
 // syndromes 65 ms (89 without teams), one easy syndrome at d = 19 23.0 (24.1).
 //
@@ -1417,12 +1418,43 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, 4) trunc_kernel(TruncArgs
         if (idx >= units) break;
         Unit<T> u{a, S, job, arena, base, base + a.caps.mps, base + 2 * a.caps.mps,
                   base + 2 * a.caps.mps + a.caps.q};
-        u.run(a.in_list ? a.in_list[idx] : (int64_t)idx);
+        u.run(a.in_list ? a.in_list[idx]
+                        : a.order ? 2 * a.order[idx >> 1] + (int64_t)(idx & 1) : (int64_t)idx);
     }
     if constexpr (T > 1) {
         if (lane == 0) job->kind = kQuit;
         team_barrier<T>();
     }
+}
+
+// Syndromes by weight, heaviest first. A unit's time follows the ranks of its
+// boundary states, which follow the syndrome's weight; a queue that hands out
+// the long units first has no long one left to start when the others are done.
+// One block: a pass to count the weights, one to place the syndromes.
+constexpr int kOrderThreads = 1024, kOrderBins = kMaxD * kMaxD;
+__device__ __forceinline__ int syndrome_weight(const uint64_t* s, int words) {
+    int w = 0;
+    for (int i = 0; i < words; ++i) w += __popcll(s[i]);
+    return w < kOrderBins ? w : kOrderBins - 1;     // (bits past the last check are the caller's)
+}
+__global__ void __launch_bounds__(kOrderThreads) order_kernel(const uint64_t* syn, int64_t B, int words,
+                                                              int64_t* order) {
+    __shared__ unsigned bin[kOrderBins];
+    for (int i = threadIdx.x; i < kOrderBins; i += kOrderThreads) bin[i] = 0;
+    __syncthreads();
+    for (int64_t b = threadIdx.x; b < B; b += kOrderThreads) atomicAdd(&bin[syndrome_weight(syn + b * words, words)], 1u);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned at = 0;
+        for (int i = kOrderBins - 1; i >= 0; --i) {
+            const unsigned n = bin[i];
+            bin[i] = at;
+            at += n;
+        }
+    }
+    __syncthreads();
+    for (int64_t b = threadIdx.x; b < B; b += kOrderThreads)
+        order[atomicAdd(&bin[syndrome_weight(syn + b * words, words)], 1u)] = b;
 }
 
 // Warps of a unit's team: the SM's sixteen, shared by the units its arenas
@@ -1464,6 +1496,11 @@ int trunc_blocks_per_sm(int arena) {
         case 2: return trunc::resident<2>(bytes);
     }
     return trunc::resident<1>(bytes);
+}
+
+bool launch_order(const uint64_t* syn, int64_t B, int words, int64_t* order, cudaStream_t s) {
+    trunc::order_kernel<<<1, trunc::kOrderThreads, 0, s>>>(syn, B, words, order);
+    return cudaGetLastError() == cudaSuccess;
 }
 
 bool launch_trunc(const TruncArgs& a, int blocks, cudaStream_t s) {

@@ -48,6 +48,7 @@ struct TruncArgs {
     TruncCaps caps;                  // shape and slice capacities of this pass
     float* ws;                       // per-unit global slices of caps.slice() floats
     unsigned long long* next_unit;   // work queue head (zeroed before the launch)
+    const int64_t* order;            // the order to take the syndromes in (nullptr: as they come)
     const int64_t* in_list;          // units to decode (nullptr: all 2B units)
     const int* in_count;             // number of entries of in_list
     int64_t* ovf_list;               // units whose shapes exceed the capacities
@@ -62,5 +63,8 @@ int trunc_units_per_block(int arena);
 size_t trunc_smem_bytes(int arena);
 int trunc_blocks_per_sm(int arena);
 bool launch_trunc(const TruncArgs& a, int blocks, cudaStream_t s);
+
+// order[B]: the syndromes by weight, heaviest first (B < 2^32).
+bool launch_order(const uint64_t* syn, int64_t B, int words, int64_t* order, cudaStream_t s);
 
 }  // namespace mld
