@@ -62,7 +62,7 @@ def kernel_sources_sha():
 
 
 def _measured_peaks():
-    """The driver-written measured peaks of this machine's GPUs, if present."""
+    """Measured peaks of the GPU, where they are recorded."""
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
             return json.load(f)
