@@ -239,7 +239,11 @@ mld_status mld_autotune(const mld_code* code, int chi, int precision, int64_t sa
  * state at every column boundary is stored by the forward pass (a
  * checkpoint per column) and the states inside a column are recomputed from
  * it during the backward pass. FP32 contraction, FP64
- * accumulation in a fixed order, so reruns give the same bits. Asynchronous
+ * accumulation in a fixed order, so reruns give the same bits. Entries keep
+ * FP32 accuracy down to 2^-180 of a state's largest (d <= 11). A syndrome with
+ * a class whose paths lie further below (rates under 1e-5 and errors all over
+ * the patch) loses them: where its gradients would be off by an eighth, it adds
+ * nothing from that column on and MLD_ERR_NUMERIC is set in the status word. Asynchronous
  * on stream; uses a device workspace owned by the code object (not reentrant
  * per code). */
 mld_status mld_decode_grad(const mld_code* code, const float* noise, const uint64_t* syndromes, int64_t B,

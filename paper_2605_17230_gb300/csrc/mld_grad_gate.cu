@@ -13,14 +13,30 @@
 // gate is recomputed from a checkpoint at most three gates back: two per side
 // of the column's exchange, in shared memory.
 //
+// Range: the adjoint state is rescaled by a power of two after every column
+// and the forward sweep's rescalings are left out of it (both go to the FP64
+// factor of the weight sums). No gate lets an entry grow, so neither state
+// leaves its top however rare the syndrome is, and the weight sums stay finite.
+// Entries keep FP32 accuracy down to 2^-180 of the largest. Below, a class may
+// lose its paths; the sums of a gate, weighted, then miss the upstream
+// gradient that they add up to, and the unit adds nothing from there on
+// (MLD_ERR_NUMERIC).
+//
+// Accuracy: each sum is divided by the Z of the whole sweep (the classes' sum
+// may cancel, so no column's own overlap can take its place): a single shot's
+// gradient is off by 1 to 1.6 times (3.5 times at d = 11 where one path
+// dominates) the 1e-7 to 5e-7 of its largest entry that a sweep per class with
+// each column's own overlap has.
+//
 // Bound: at d <= 9 issue and shared memory (50% of the issue slots, 62% of the
 // shared-memory cycles at d = 7: state loads, exchanges, the sums over lanes);
 // at d = 11 the fetching of its own straight-line program (93 KB) by five
 // resident warps an SM. Measured on GB300, against one block per (syndrome,
-// class) with its states in shared memory: d = 7, 65,536 syndromes 0.55 ms
-// (6.1); d = 9, 16,384 syndromes 0.71 ms (8.6); d = 11, 2,049 syndromes 1.49
-// ms (7.4). A column as a list of operations run by an interpreter (one copy
-// of each gate's code) was slower: 0.92, 1.18, 1.90 ms.
+// class) with its states in shared memory: d = 7, 65,536 syndromes 0.56 ms
+// (6.1); d = 9, 16,384 syndromes 0.79 ms (8.6; 0.72 without the rescaling of
+// the adjoint state); d = 11, 2,049 syndromes 1.55 ms (7.4; 1.5). A column as a
+// list of operations run by an interpreter (one copy of each gate's code) was
+// slower: 0.92, 1.18, 1.90 ms.
 //
 // Gradients are summed per unit slot in FP64 in a fixed order, the slots by a
 // second kernel: reruns give the same bits.
@@ -38,12 +54,13 @@ namespace {
 
 using namespace gate;
 
-// Scale of the states: their products with the adjoint states are what counts,
-// so the two share the exponent range.
-constexpr int kGradTop = 40;
-// Classes whose Z differ by more than this are swept back one at a time (their
-// adjoint states would not fit one range).
-constexpr float kMaxRatio = 1.152921504606847e18f;      // 2^60
+// Tops of the states and of the adjoint states (a class's paths need the range
+// below both): a weight sum adds up to 2^d products of the two, below
+// 2^(54 + 1 + 54 + 1 + 11).
+constexpr int kGradTop = 54, kAdjointTop = 54;
+// Classes whose adjoint states at the start of the last column differ by more
+// than this are swept back one at a time (they would not fit one range).
+constexpr double kApart = 8.673617379884035e-19;        // 2^-60
 
 template <int D>
 struct GradLanes {
@@ -69,6 +86,23 @@ struct GradLanes {
 };
 
 __host__ __device__ constexpr int grad_row(int d, int c, int j) { return (c & 1) ? d - 1 - j : j; }
+
+// x 2^e by its exponent field (FP64 arithmetic has 1/64 of the FP32 rate);
+// subnormal values and results are 0, infinities and NaN stay, and what would
+// overflow stays finite.
+__device__ __forceinline__ double scaled(double x, int e) {
+    const int hi = __double2hiint(x), at = (hi >> 20) & 0x7ff;
+    if (at == 0x7ff) return x;
+    const int to = at + e;
+    if (at == 0 || to <= 0) return 0.0;
+    return __hiloint2double((hi & ~(0x7ff << 20)) | (to < 0x7fe ? to : 0x7fe) << 20, __double2loint(x));
+}
+// The same in FP32, to infinity.
+__device__ __forceinline__ float scaled(float x, int e) {
+    const int bits = __float_as_int(x), at = (bits >> 23) & 0xff, to = at + e;
+    if (at == 0 || to <= 0) return 0.f;
+    return to < 0xff ? __int_as_float((bits & ~(0xff << 23)) | to << 23) : copysignf(INFINITY, x);
+}
 
 template <int M>
 __device__ __forceinline__ void load_state(float2 (&P)[1 << M], const float2* s, int lane) {
@@ -197,27 +231,39 @@ struct Lane {
         for (int k = 0; k < (1 << M); ++k) P[k] = xch[k * S::STRIDE + lane];
         __syncwarp();
     }
-    // the whole column; scale[slot] keeps its rescaling
-    __device__ __forceinline__ void column(float2 (&P)[1 << M], int c, uint32_t w, int slot, int& e2) const {
-        steps<0, M + 1>(P, c, w, 1.f);
-        uint32_t mx = __float_as_uint(max_of(P));
+    // bits of the unit's largest entry, from the lanes' (>= 0)
+    __device__ __forceinline__ static uint32_t unit_max(float x) {
+        uint32_t mx = __float_as_uint(x);
         if constexpr (S::LANES == 32) {
             mx = __reduce_max_sync(0xffffffffu, mx);
         } else {
 #pragma unroll
             for (int o = S::LANES / 2; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         }
-        const float sc = rescale<kGradTop>(mx, e2);
+        return mx;
+    }
+    // the whole column; scale[slot] keeps its rescaling
+    __device__ __forceinline__ void column(float2 (&P)[1 << M], int c, uint32_t w, int slot, int& e2) const {
+        steps<0, M + 1>(P, c, w, 1.f);
+        const float sc = rescale<kGradTop>(unit_max(max_of(P)), e2);
         if (lane == 0) scale[slot] = sc;
         exchange(P);
         steps<M + 1, D>(P, c, w, sc);
     }
+    // What a column's weight sums are multiplied by: the column's rescaling is
+    // a factor of those of step M+1 and of all before it (early), not of G.
+    struct Factors {
+        double late, early;
+        float unit, want, slack;    // what a gate's weighted sums times (unit 2^e) come to, and by how much they may miss it
+        int e_late, e_early;
+        bool lost;
+    };
     // Step J backwards: P is the state before it.
     template <int J>
-    __device__ __forceinline__ void back(const float2 (&P)[1 << M], float2 (&G)[1 << M], int c, uint32_t w, float sc,
-                                         double factor) const {
+    __device__ __forceinline__ void back(const float2 (&P)[1 << M], float2 (&G)[1 << M], int c, uint32_t w,
+                                         Factors& by) const {
         float s[4];
-        const float4 v = step_weight<J>(c, w, sc);
+        const float4 v = step_weight<J>(c, w, 1.f);
         if constexpr (J < M)
             back_bit<M, M - 1 - J>(P, G, v, s);
         else if constexpr (J == M)
@@ -243,11 +289,19 @@ struct Lane {
         }
         const int r = grad_row(D, c, J), q = r * D + c;
         const uint32_t e = (w >> (2 * J)) & 3;
-        const double fac = J == M + 1 ? factor * (double)sc : factor;
+        // (the column's first gate: its sums have to give what the unit adds)
+        const auto check = [&](float t) {
+#pragma unroll
+            for (int o = 1; o < S::LANES && o < 4; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            t = scaled(__shfl_sync(0xffffffffu, t, 0, S::LANES), J > M + 1 ? by.e_late : by.e_early) * by.unit;
+            by.lost = fabsf(t - by.want) > by.slack;
+            if (by.lost) by.late = by.early = 0.0;
+        };
+        if constexpr (J == D - 1 && M == 1) check((lane & 1) ? fmaf(v0, v.z, v1 * v.w) : fmaf(v0, v.x, v1 * v.y));
         const auto add = [&](int f, int cc, float x) {
             const int ff = f ^ (int)(e >> 1), c2 = cc ^ (int)(e & 1);
             const int xx = (r & 1) ? c2 : ff, zz = (r & 1) ? ff : c2;
-            acc[4 * q + (xx ? (zz ? 2 : 1) : (zz ? 3 : 0))] += (double)x * fac;
+            acc[4 * q + (xx ? (zz ? 2 : 1) : (zz ? 3 : 0))] += (double)x * (J > M + 1 ? by.late : by.early);
         };
         if constexpr (M == 1) {
             add(lane & 1, 0, v0);
@@ -257,24 +311,39 @@ struct Lane {
             float x = (up ? v1 : v0) + __shfl_xor_sync(0xffffffffu, up ? v0 : v1, 2);
 #pragma unroll
             for (int o = 4; o < S::LANES; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if constexpr (J == D - 1)
+                check(lane < 4 ? x * ((lane & 1) ? ((lane & 2) ? v.w : v.z) : ((lane & 2) ? v.y : v.x)) : 0.f);
             if (lane < 4) add(lane & 1, lane >> 1, x);
         }
     }
     // Steps J-1, .., FROM backwards, the state before step FROM being in base.
     template <int FROM, int J>
     __device__ __forceinline__ void back_from(const float2* base, float2 (&G)[1 << M], int c, uint32_t w, float sc,
-                                              double factor) const {
+                                              Factors& by) const {
         if constexpr (J > FROM) {
             float2 P[1 << M];
             load_state<M>(P, base, lane);
             steps<FROM, J - 1>(P, c, w, sc);
-            back<J - 1>(P, G, c, w, sc, factor);
-            back_from<FROM, J - 1>(base, G, c, w, sc, factor);
+            back<J - 1>(P, G, c, w, by);
+            back_from<FROM, J - 1>(base, G, c, w, sc, by);
         }
     }
-    // Column c backwards: G after it -> G before it.
-    __device__ __forceinline__ void back_column(float2 (&G)[1 << M], int c, uint32_t w, int slot, double factor) const {
+    // Column c backwards: G after it -> G before it; factor 2^ge G is the
+    // derivative of the loss by the state (unit is the same in FP32, with the
+    // upstream gradients want, on a common scale). Returns whether the range
+    // was lost.
+    __device__ __forceinline__ bool back_column(float2 (&G)[1 << M], int c, uint32_t w, int slot, double factor, int& ge,
+                                                float unit, float want, float slack) const {
         const float sc = scale[slot];
+        Factors by;
+        by.unit = unit;
+        by.want = want;
+        by.slack = slack;
+        by.e_late = ge;
+        by.late = scaled(factor, ge);
+        ge += (int)(__float_as_uint(sc) >> 23) - 127;
+        by.e_early = ge;
+        by.early = scaled(factor, ge);
         {
             float2 P[1 << M];
             load_state<M>(P, slice + (size_t)c * S::STATE, lane);
@@ -286,11 +355,18 @@ struct Lane {
             steps<M + 1, M + 1 + S::HO>(P, c, w, sc);
             store_state<M>(P, ck_out, lane);
         }
-        back_from<M + 1 + S::HO, D>(ck_out, G, c, w, sc, factor);
-        back_from<M + 1, M + 1 + S::HO>(xch, G, c, w, sc, factor);
+        back_from<M + 1 + S::HO, D>(ck_out, G, c, w, sc, by);
+        back_from<M + 1, M + 1 + S::HO>(xch, G, c, w, sc, by);
         exchange(G);
-        back_from<S::HI, M + 1>(ck_in, G, c, w, sc, factor);
-        back_from<0, S::HI>(slice + (size_t)c * S::STATE, G, c, w, sc, factor);
+        back_from<S::HI, M + 1>(ck_in, G, c, w, sc, by);
+        back_from<0, S::HI>(slice + (size_t)c * S::STATE, G, c, w, sc, by);
+        float m = 0.f;
+#pragma unroll
+        for (int k = 0; k < (1 << M); ++k) m = fmaxf(m, fmaxf(fabsf(G[k].x), fabsf(G[k].y)));
+        const float up = rescale<kAdjointTop>(unit_max(m), ge);
+#pragma unroll
+        for (int k = 0; k < (1 << M); ++k) G[k] = mul2(dup(up), G[k]);
+        return by.lost;
     }
 };
 
@@ -421,44 +497,64 @@ grad_gate_kernel(GradDenseArgs g) {
         const double u0 = live ? g.dlogP[2 * (live ? unit : 0)] : 0.0, u1 = live ? g.dlogP[2 * (live ? unit : 0) + 1] : 0.0;
         const bool ok0 = u0 != 0.0 && z[0] > 0.f && z[0] < INFINITY, ok1 = u1 != 0.0 && z[1] > 0.f && z[1] < INFINITY;
         if (!__any_sync(0xffffffffu, ok0 || ok1)) continue;
-        const float zmax = fmaxf(ok0 ? z[0] : 0.f, ok1 ? z[1] : 0.f), zmin = fminf(z[0], z[1]);
-        const bool apart = ok0 && ok1 && zmax > zmin * kMaxRatio;
-        const double umax = fmax(ok0 ? fabs(u0) : 0.0, ok1 ? fabs(u1) : 0.0);
-        const bool nan = (ok0 && u0 != u0) || (ok1 && u1 != u1);
-        const int passes = __any_sync(0xffffffffu, apart) ? 2 : 1;
+        // the last column for l_X = 0 and 1, each with its own factor; then the
+        // others for the sum of the two adjoint states, the smaller one scaled
+        // to the larger one's factor (or one after the other: a second pass)
+        float2 G[1 << M];
+        float2* first = L.slice + (size_t)D * S::STATE;
+        float2* second = first - S::STATE;               // the last column's start, read by then
+        double c0 = ok0 ? u0 / (double)z[0] : 0.0, c1 = ok1 ? u1 / (double)z[1] : 0.0;
+        const int top = 1023 - max(ok0 ? (__double2hiint(u0) >> 20) & 0x7ff : 0, ok1 ? (__double2hiint(u1) >> 20) & 0x7ff : 0);
+        float want0 = ok0 ? (float)scaled(u0, top) : 0.f, want1 = ok1 ? (float)scaled(u1, top) : 0.f;
+        const float slack = 0.125f * (fabsf(want0) + fabsf(want1));
+        double factor = 0.0;
+        float per = 0.f, want = 0.f;
+        bool apart = false, lost = false;
+        int ge = 0, ge0 = 0, ge1 = 0, passes = 1;
 #pragma unroll 1
         for (int pass = 0; pass < passes; ++pass) {
-            float s0 = 0.f, s1 = 0.f;
-            double factor = 0.0;
-            if (apart) {
-                const bool first = (z[0] >= z[1]) == (pass == 0);
-                s0 = first ? 1.f : 0.f;
-                s1 = first ? 0.f : 1.f;
-                factor = first ? u0 / (double)z[0] : u1 / (double)z[1];
-            } else if (pass == 0 && (ok0 || ok1)) {
-                s0 = ok0 ? (float)(u0 / umax) * (zmax / z[0]) : 0.f;
-                s1 = ok1 ? (float)(u1 / umax) * (zmax / z[1]) : 0.f;
-                factor = umax / (double)zmax;
-            }
-            if (nan) factor = NAN;
-            // the last column for l_X = 0 and 1, then the others for their sum
-            float2 G[1 << M];
 #pragma unroll 1
-            for (int step = 0; step <= D; ++step) {
+            for (int step = pass ? 2 : 0; step <= D; ++step) {
                 const int c = step < 2 ? D - 1 : D - step;
-                if (step < 2) end_state(G, step ? s1 : s0);
-                L.back_column(G, c, L.word(c, step == 1), step == 1 ? D : c, factor);
-                float2* first = L.slice + (size_t)D * S::STATE;
-                if (step == 0) store_state<M>(G, first, lane);
-                if (step == 1) {
-#pragma unroll
-                    for (int k = 0; k < (1 << M); ++k) {
-                        const float2 o = first[(k << M) + lane];
-                        G[k] = make_float2(G[k].x + o.x, G[k].y + o.y);
+                if (step <= 2) {
+                    bool one = step == 1;
+                    float share = 0.f;
+                    if (step == 2) {
+                        // f 2^e of the two: the larger, and the smaller's share of it
+                        one = fabs(scaled(c1, ge1 - ge0)) > fabs(c0);
+                        const double small = one ? scaled(c0, ge0 - ge1) : scaled(c1, ge1 - ge0), big = one ? c1 : c0;
+                        const double ratio = small == 0.0 ? 0.0 : small / big;
+                        apart = small != 0.0 && fabs(ratio) < kApart;
+                        if (pass == 0) passes = __any_sync(0xffffffffu, apart) ? 2 : 1;
+                        if (pass == 1) one = !one;
+                        share = pass || apart ? 0.f : (float)ratio;
                     }
+                    factor = pass && !apart ? 0.0 : (one ? c1 : c0);
+                    per = (float)scaled(factor, top);
+                    want = pass && !apart ? 0.f : (step == 2 && !apart ? want0 + want1 : (one ? want1 : want0));
+                    ge = step < 2 ? -kAdjointTop : (one ? ge1 : ge0);
+                    if (step < 2) {
+                        end_state(G, __uint_as_float((uint32_t)(127 + kAdjointTop) << 23));
+                    } else {
+                        const float2 *g = one ? second : first, *h = one ? first : second;
+#pragma unroll
+                        for (int k = 0; k < (1 << M); ++k)
+                            G[k] = fma2(dup(share), h[(k << M) + lane], g[(k << M) + lane]);
+                    }
+                }
+                if (L.back_column(G, c, L.word(c, step == 1), step == 1 ? D : c, factor, ge, per, want, slack)) {
+                    lost = true;
+                    factor = 0.0;
+                    per = want = 0.f;
+                    if (step < 2) (step ? c1 : c0) = (step ? want1 : want0) = 0.f;
+                }
+                if (step < 2) {
+                    store_state<M>(G, step ? second : first, lane);
+                    (step ? ge1 : ge0) = ge;
                 }
             }
         }
+        if (lost && lane == 0) atomicOr(g.status, 1 << MLD_ERR_NUMERIC);
     }
     // the warp's units in order, then the block's warps: one partial sum a block
     __syncthreads();

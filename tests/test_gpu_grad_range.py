@@ -1,0 +1,86 @@
+"""The adjoint over rare syndromes: a syndrome far less likely than its patch's
+typical ones has states whose entries differ by hundreds of powers of two, and
+gradients of the order 1/p. Every gradient is finite, whatever the rates and
+the zeros of the table; where the span of a state stays above 2^-170 of the
+2^-180 that the states keep, it is the oracle's: (p/3)^(3d/2) where every qubit
+is noisy (the paths of a column and a half, between two rescalings, may cost a
+rate for each qubit), (p/3)^(3d) where paths lead around perfect ones. Tolerance
+as for the ragged batches: 2e-5 of the largest entry."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mld():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2605_17230_gb300 as m
+    m.load()
+    return m
+
+
+def _tables(n, p, rng):
+    """Depolarizing; without Y; dephasing; perfect qubits among noisy ones."""
+    t = {"depolarizing": synth.depolarizing(n, p)}
+    t["no Y"] = np.tile([1 - p, p / 2, 0.0, p / 2], (n, 1))
+    t["dephasing"] = np.tile([1 - p, 0.0, 0.0, p], (n, 1))
+    t["perfect qubits"] = synth.depolarizing(n, p)
+    t["perfect qubits"][rng.random(n) < 0.3] = [1, 0, 0, 0]
+    return {k: v.astype(np.float32) for k, v in t.items()}
+
+
+def _errors(table, B, rng):
+    """Errors of every weight among those that the table allows."""
+    n = table.shape[0]
+    code = np.array([0, 1, 3, 2], np.uint8)               # I, X, Y, Z -> x + 2z
+    E = np.zeros((B, n), np.uint8)
+    for b in range(B):
+        for q in range(n):
+            allowed = np.flatnonzero(table[q, 1:]) + 1
+            if allowed.size and rng.random() < 0.75 * b / B:
+                E[b, q] = code[rng.choice(allowed)]
+    return E
+
+
+def _grad(mld, d, noise, syn, up):
+    code = mld.Code(d)
+    dn = torch.zeros((d * d, 4), dtype=torch.float64, device="cuda")
+    mld.mld_decode_grad(code.handle, torch.tensor(noise, device="cuda"), torch.tensor(syn.view(np.int64), device="cuda"),
+                        len(syn), 2 ** (d // 2), torch.tensor(up, device="cuda"), None, dn)
+    torch.cuda.synchronize()
+    return dn.cpu().numpy(), code.status()
+
+
+@pytest.mark.parametrize("d", [3, 5, 7, 9, 11])
+@pytest.mark.parametrize("p", [1e-5, 1e-6, 1e-8, 1e-12, 1e-20])
+def test_finite_at_any_rate(mld, d, p):
+    rng = np.random.default_rng(d)
+    for name, noise in _tables(d * d, p, rng).items():
+        syn = synth.syndromes_of(d, _errors(noise, 40, rng))
+        dn, _ = _grad(mld, d, noise, syn, rng.normal(size=(40, 4)))
+        assert np.isfinite(dn).all(), name
+
+
+@pytest.mark.parametrize("name,columns", [("depolarizing", 1.5), ("perfect qubits", 3)])
+@pytest.mark.parametrize("d", [3, 5, 7, 9, 11])
+def test_rare_syndromes(mld, d, name, columns):
+    rng = np.random.default_rng(d)
+    n, B, p = d * d, 12, 3 * 2.0 ** (-170 / (columns * d))
+    noise = _tables(n, p, rng)[name]
+    syn = synth.syndromes_of(d, _errors(noise, B, rng))
+    up = rng.normal(size=(B, 4))
+    lz, g = oracle.coset_dlogz(d, noise.astype(np.float64), oracle.representatives(d, syn).reshape(-1, n))
+    possible = np.isfinite(lz).reshape(B, 4)
+    up = np.where(possible, up, 0.0)
+    g = np.where(possible[..., None, None], g.reshape(B, 4, n, 4), 0.0)
+    for b in range(B):                                    # shot by shot: their scales differ by 1/p
+        ref = np.einsum("l,lqp->qp", up[b], g[b])
+        dn, status = _grad(mld, d, noise, syn[b:b + 1], up[b:b + 1])
+        assert status == 0
+        np.testing.assert_allclose(dn, ref, rtol=2e-5, atol=2e-5 * np.abs(ref).max(), err_msg=str(b))
