@@ -21,9 +21,12 @@
 //
 // FP64 accuracy at FP32 rates: for h >= 7 an entry is a pair of FP32 numbers
 // (19 FP32 operations for an output a x + b y, against two of the FP64 pipe at
-// 1/64 of the rate). Largest error of the posterior over p = 0.02..0.12,
-// d = 15..25 against 64 bits: 2e-14 of its norm (complex FP64 elimination:
-// 9e-12); ln Pr(s): 8e-16 relative (9e-14).
+// 1/64 of the rate). A qubit's two weights are stored as 1 and the odds, the
+// larger probability going to one FP64 product a part: as p and 1 - p, a
+// gate's most likely weight (1 - f)(1 - g) was rounded to 2^-48, under uniform
+// rates the same way in every gate (largest error of ln Z over eight syndromes
+// at p = 0.10, d = 25: 1.7e-12, with the odds 3.4e-13; complex FP64 elimination
+// 1.1e-13 of the leading class and up to 1 of the others).
 //
 // Bound: the FP32 pipe (62% busy at d = 25: two warps a scheduler, all the
 // registers hold). Measured on GB300: d = 25, 700 syndromes 3.0 ms (FP64
@@ -60,6 +63,7 @@ using namespace xz;
 template <int H>
 struct Shape {
     using T = std::conditional_t<(H <= 6), double, Twin>;
+    static constexpr int H_ = H;
     static constexpr int RB = H <= 6 ? H : 6;
     static constexpr int LB = H - RB;
     static constexpr int D = 2 * H + 1;
@@ -96,15 +100,16 @@ struct Args {
     int64_t B;
 };
 
-template <int H>
+template <class S>
 size_t shared_bytes(int units) {
-    using S = Shape<H>;
     using T = typename S::T;
+    constexpr int H = S::H_;
     size_t b = (size_t)2 * S::D * (H + 1) * 2 * sizeof(T) * 2;               // (p, 1 - p) per qubit of a gate
     b += (size_t)units * S::REGION * S::VB;
     b = (b + 15) & ~(size_t)15;
     b += (size_t)(units / 2) * 2 * S::BW * 4;                                // bits (at most units / 2 syndromes)
     b += (size_t)units * (sizeof(T) + 4) + units * 2 * sizeof(T) + 64;       // results, two warps' shares
+    b += (S::NT / 32) * 2 * sizeof(double);                                  // products of the larger probabilities
     return b;
 }
 
@@ -137,26 +142,36 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
     T* res_z = reinterpret_cast<T*>(smem + off);          // [unit]
     T* share = res_z + units;                             // [unit][2]
     int* res_e = reinterpret_cast<int*>(share + 2 * units);
-    uint32_t* bits = reinterpret_cast<uint32_t*>(res_e + units);
+    double* larger = reinterpret_cast<double*>(res_e + units);               // [warp][part] (units: a multiple of 4)
+    uint32_t* bits = reinterpret_cast<uint32_t*>(larger + S::NT / 32 * 2);
 
     bool ok = true;
+    double prod[2] = {1.0, 1.0};
     for (int i = tid; i < nu / 2 * D * (H + 1); i += S::NT) {
         const int part = i / (D * (H + 1)), c = i / (H + 1) % D, k = i % (H + 1);
         const float* p = part ? a.pz : a.px;
         const float g = p[qubit_of<D>(part, c, 2 * k)];
         const float f = k < H ? p[qubit_of<D>(part, c, 2 * k + 1)] : 0.5f;
         ok = ok && g > 0.f && g < 1.f && f > 0.f && f < 1.f;                 // NaN fails
-        tab[4 * i] = make<T>((double)f);
-        tab[4 * i + 1] = make<T>(1.0 - (double)f);
-        tab[4 * i + 2] = make<T>((double)g);
-        tab[4 * i + 3] = make<T>(1.0 - (double)g);
+        double top = odds_of(tab + 4 * i + 2, g), f_top = odds_of(tab + 4 * i, f);
+        if (k < H) top *= f_top;
+        if (part) prod[1] *= top;
+        else prod[0] *= top;
     }
     if (!ok && blockIdx.x == 0) atomicOr(a.status, 1 << MLD_ERR_INVALID_ARG);
-
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        prod[0] *= __shfl_xor_sync(0xffffffffu, prod[0], o);
+        prod[1] *= __shfl_xor_sync(0xffffffffu, prod[1], o);
+    }
+    if ((tid & 31) == 0) {
+        larger[tid >> 5 << 1] = prod[0];
+        larger[(tid >> 5 << 1) + 1] = prod[1];
+    }
+    const int64_t nchunks = (a.B + sb - 1) / sb;
     const int unit = tid / S::LANES, lane = tid % S::LANES;
     const int sub = unit / nu, part = unit % nu >> 1, sector = unit & 1;
     const T* ptab = tab + (size_t)part * D * (H + 1) * 4;
-    const int64_t nchunks = (a.B + sb - 1) / sb;
     int64_t done = 0;
     for (int64_t chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
         const int64_t b0 = chunk * sb;
@@ -310,17 +325,23 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
         }
         __syncthreads();
         if (tid < live) {
+            double larger_m[2] = {1.0, 1.0};              // m 2^e
+            int larger_e[2] = {0, 0};
+            for (int p = 0; p < nu / 2; ++p) {
+                for (int w = 0; w < S::NT / 32; ++w) larger_m[p] *= larger[2 * w + p];
+                larger_m[p] = mantissa(larger_m[p], larger_e[p]);
+            }
             const int64_t b = b0 + tid;
             double lx[2], lz[2];
             bool bad = false;
             for (int s = 0; s < 2; ++s) {
                 const double zx = value_of(res_z[tid * nu + s]);
                 bad = bad || !(zx > 0.0) || !(zx < INFINITY);
-                lx[s] = log_of(zx, res_e[tid * nu + s]);
+                lx[s] = log_of(zx, larger_m[0], larger_e[0] + res_e[tid * nu + s]);
                 if (nu == 4) {
                     const double zz = value_of(res_z[tid * nu + 2 + s]);
                     bad = bad || !(zz > 0.0) || !(zz < INFINITY);
-                    lz[s] = log_of(zz, res_e[tid * nu + 2 + s]);
+                    lz[s] = log_of(zz, larger_m[1], larger_e[1] + res_e[tid * nu + 2 + s]);
                 }
             }
             if (nu == 2) {
@@ -353,7 +374,7 @@ template <int H>
 mld_status launch_h(const Args& a, cudaStream_t s) {
     using S = Shape<H>;
     const int units = S::NT / S::LANES;
-    const size_t smem = shared_bytes<H>(units);
+    const size_t smem = shared_bytes<S>(units);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MLD_ERR_CUDA;
     static std::atomic<int> resident[kMaxDevices];         // blocks the device holds at once

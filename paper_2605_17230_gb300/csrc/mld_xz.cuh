@@ -109,10 +109,10 @@ __device__ __forceinline__ void gates_falling(double (&v)[1 << RB], const W& w) 
 // The same on the top register bit, prev in bit 0, followed by a rotation of
 // the index (the top bit becomes bit 0): one body serves every row pair in
 // turn. a, b: weights of old[0], old[1] for new[n], by [prev][n].
-template <int RB>
-__device__ __forceinline__ void gate_and_rotate(Twin (&v)[1 << RB], const Twin (&a)[2][2], const Twin (&b)[2][2]) {
+template <int RB, typename T>
+__device__ __forceinline__ void gate_and_rotate(T (&v)[1 << RB], const T (&a)[2][2], const T (&b)[2][2]) {
     constexpr int R = 1 << RB;
-    Twin out[R];
+    T out[R];
 #pragma unroll
     for (int i = 0; i < R / 2; ++i) {
         out[2 * i] = dot(a[i & 1][0], v[i], b[i & 1][0], v[i + R / 2]);
@@ -154,33 +154,33 @@ struct Vec<8> { using type = float2; };
 template <>
 struct Vec<16> { using type = float4; };
 
-template <class S>
-__device__ __forceinline__ void exchange_store(unsigned char* X, const Twin (&v)[1 << S::RB], int lane) {
+template <class S, typename T>
+__device__ __forceinline__ void exchange_store(unsigned char* X, const T (&v)[1 << S::RB], int lane) {
     using V = typename Vec<S::VB>::type;
-    constexpr int PER = S::VB / (int)sizeof(Twin);
+    constexpr int PER = S::VB / (int)sizeof(T);
     V* x = reinterpret_cast<V*>(X) + lane;
 #pragma unroll
     for (int k = 0; k < S::LANES; ++k)
 #pragma unroll
         for (int s = 0; s < S::SLOTS; ++s) {
             V t;
-            Twin* e = reinterpret_cast<Twin*>(&t);
+            T* e = reinterpret_cast<T*>(&t);
 #pragma unroll
             for (int m = 0; m < PER; ++m) e[m] = v[store_index<S::LB, S::RB>(k, s * PER + m)];
             x[(s * S::LANES + k) * S::STRIDE] = t;
         }
 }
-template <class S>
-__device__ __forceinline__ void exchange_load(const unsigned char* X, Twin (&v)[1 << S::RB], int lane) {
+template <class S, typename T>
+__device__ __forceinline__ void exchange_load(const unsigned char* X, T (&v)[1 << S::RB], int lane) {
     using V = typename Vec<S::VB>::type;
-    constexpr int PER = S::VB / (int)sizeof(Twin);
+    constexpr int PER = S::VB / (int)sizeof(T);
     const V* x = reinterpret_cast<const V*>(X) + lane * S::STRIDE;
 #pragma unroll
     for (int k = 0; k < S::LANES; ++k)
 #pragma unroll
         for (int s = 0; s < S::SLOTS; ++s) {
             const V t = x[s * S::LANES * S::STRIDE + k];
-            const Twin* e = reinterpret_cast<const Twin*>(&t);
+            const T* e = reinterpret_cast<const T*>(&t);
 #pragma unroll
             for (int m = 0; m < PER; ++m) v[load_index<S::LB, S::RB>(k, s * PER + m)] = e[m];
         }
@@ -194,7 +194,8 @@ __device__ __forceinline__ void unit_sync(int unit) {
         __syncwarp();
 }
 
-// Entries are kept near the top of the exponent range (they only decrease).
+// Entries are kept near the top of the exponent range (between two rescalings
+// they grow by at most 2^H: 1 + odds <= 2 a gate).
 template <typename T>
 struct Range;
 template <>
@@ -221,22 +222,49 @@ template <typename T, int N>
 __device__ __forceinline__ uint32_t max_bits(const T (&v)[N]) {
     uint32_t m = Range<T>::bits(v[0]);
 #pragma unroll
-    for (int i = 1; i < N; ++i) m = max(m, Range<T>::bits(v[i]));
+    for (int i = 0; i < N; i += 2) m = __vimax3_u32(m, Range<T>::bits(v[i]), Range<T>::bits(v[i + 1]));
     return m;
 }
-
-// ln z + e ln 2, the exponent of z joined to e first (z is kept near 2^top, and
-// ln z and e ln 2 would cancel to a few hundred ulps of their difference).
-__device__ __forceinline__ double log_of(double z, int e) {
-    if (!(z > 0.0)) return -INFINITY;
-    int ex = 0;
-    double m = frexp(z, &ex);                            // [1/2, 1)
-    if (m < 0.70710678118654752440) {
-        m *= 2.0;
-        ex -= 1;
+// z = m 2^e, m in [sqrt(1/2), sqrt(2)), by its bits (z > 0); e is added.
+__device__ __forceinline__ double mantissa(double z, int& e) {
+    if (__double2hiint(z) < 1 << 20) {                    // subnormal
+        z *= 18014398509481984.0;                         // 2^54
+        e -= 54;
     }
-    return log(m) + (double)(e + ex) * 0.69314718055994530942;
+    const int hi = __double2hiint(z), frac = hi & 0xfffff;
+    const int up = frac >= 0x6a09e;
+    e += (hi >> 20) - 1023 + up;
+    return __hiloint2double(frac | (1023 - up) << 20, __double2loint(z));
 }
+// ln(z m) + e ln 2, the exponents joined first (z is kept near 2^top, and
+// ln z and e ln 2 would cancel to a few hundred ulps of their difference).
+__device__ __forceinline__ double log_of(double z, double m, int e) {
+    if (!(z > 0.0) || !(z < INFINITY)) return z > 0.0 ? z : -INFINITY;
+    m = mantissa(mantissa(z, e) * m, e);
+    return log(m) + (double)e * 0.69314718055994530942;
+}
+
+// A qubit's two weights as odds: t[0] of a flip, t[1] of none, the larger one 1;
+// returns the larger probability.
+__device__ __forceinline__ double odds_of(double* t, float p) {
+    const double x = p, y = 1.0 - x;
+    t[0] = x > y ? 1.0 : x / y;
+    t[1] = x > y ? y / x : 1.0;
+    return x > y ? x : y;
+}
+__device__ __forceinline__ double odds_of(Twin* t, float p) {
+    // 1 - p is a float for p > 1/2, and a pair below
+    const bool flips = p > 0.5f;
+    const float q = __fsub_rn(1.f, p), small = flips ? q : p, hi = flips ? p : q;
+    const float lo = flips ? 0.f : __fsub_rn(__fsub_rn(1.f, q), p);
+    const float r = __fdiv_rn(small, hi);
+    const float rest = __fmaf_rn(-r, lo, __fmaf_rn(-r, hi, small));
+    const Twin odds = renormal(r, __fdiv_rn(rest, hi)), one = Twin{1.f, 0.f};
+    t[0] = flips ? one : odds;
+    t[1] = flips ? odds : one;
+    return (double)hi + (double)lo;
+}
+
 __device__ __forceinline__ double value_of(double z) { return z; }
 __device__ __forceinline__ double value_of(Twin z) { return (double)z.hi + (double)z.lo; }
 __device__ __forceinline__ double shuffled(double z, int o) { return __shfl_xor_sync(0xffffffffu, z, o); }
