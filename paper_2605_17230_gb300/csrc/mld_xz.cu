@@ -28,10 +28,17 @@
 // at p = 0.10, d = 25: 1.7e-12, with the odds 3.4e-13; complex FP64 elimination
 // 1.1e-13 of the leading class and up to 1 of the others).
 //
+// Range: a pair has FP32's exponents. A unit watches its smallest entry at
+// every rescaling; where one lies so low that the subnormals lost since the
+// last may show, or where a rate is below 2^-33, the syndrome is marked and a
+// second pass decodes it in FP64 (rescaled alike, entries 2^1880 apart). At
+// d = 25 that is every syndrome from about p = 3e-3 down, at d = 17 from 1e-4.
+//
 // Bound: the FP32 pipe (62% busy at d = 25: two warps a scheduler, all the
-// registers hold). Measured on GB300: d = 25, 700 syndromes 3.0 ms (FP64
-// pipe instead of pairs 13.7, banded elimination 125.8); d = 17, 1,024
-// syndromes 0.22 ms (0.70, 42); d = 9, 1,024 syndromes 0.10 ms (4.9).
+// registers hold). Measured on GB300: d = 25, 700 syndromes 2.9 ms (all of
+// them in the FP64 pass as well 17; banded elimination 125.8); d = 17, 1,024
+// syndromes 0.20 ms (42; 2 us of it the second launch, which finds no mark);
+// d = 9, 1,024 syndromes 0.10 ms (4.9).
 // Registers hold RB bits of the state, lanes the rest, and a column exchanges them once
 // through shared memory. A column's program is the same in both directions:
 // at its start register bit t holds the row pair j = RB-1-t in processing
@@ -60,9 +67,10 @@ using namespace xz;
 
 // h <= 6: a thread holds the whole state in FP64, columns unrolled in pairs.
 // Above: 64 entries of twice FP32 (128 registers); 64 lanes a unit at d = 25.
-template <int H>
+template <int H, bool WIDE = false>
 struct Shape {
-    using T = std::conditional_t<(H <= 6), double, Twin>;
+    static constexpr bool kPairs = H > 6 && !WIDE;
+    using T = std::conditional_t<kPairs, Twin, double>;
     static constexpr int H_ = H;
     static constexpr int RB = H <= 6 ? H : 6;
     static constexpr int LB = H - RB;
@@ -109,7 +117,7 @@ size_t shared_bytes(int units) {
     b = (b + 15) & ~(size_t)15;
     b += (size_t)(units / 2) * 2 * S::BW * 4;                                // bits (at most units / 2 syndromes)
     b += (size_t)units * (sizeof(T) + 4) + units * 2 * sizeof(T) + 64;       // results, two warps' shares
-    b += (S::NT / 32) * 2 * sizeof(double);                                  // products of the larger probabilities
+    b += (S::NT / 32) * 2 * sizeof(double) + units * 4;                      // products of the larger probabilities, low
     return b;
 }
 
@@ -120,9 +128,16 @@ __host__ __device__ __forceinline__ int qubit_of(int part, int c, int j) {
     return part == 0 ? (D - 1 - c) * D + r : r * D + c;
 }
 
-template <int H>
+// A rate below this leaves products of three weights no room in a pair.
+constexpr float kPairRate = 1.1641532182693481e-10f;    // 2^-33
+__device__ __forceinline__ float small_rate(float p) { return p > 0.5f ? 1.f - p : p; }
+// In logP[b][0]: a syndrome for the FP64 pass.
+__device__ __forceinline__ bool is_marked(double l) { return l != l; }
+
+// WIDE: the FP64 pass over the syndromes that the pairs marked.
+template <int H, bool WIDE>
 __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
-    using S = Shape<H>;
+    using S = Shape<H, WIDE>;
     using T = typename S::T;
     constexpr int D = S::D, RB = S::RB, LB = S::LB;
     using Scale = typename ScaleOf<T>::type;
@@ -133,6 +148,12 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
     const int per = nu * S::LANES;                        // threads of a syndrome
     const int sb = S::NT / per;                           // syndromes a block decodes at a time
     const int units = S::NT / S::LANES;
+    if constexpr (WIDE) {                                 // nothing to do, as a rule
+        bool any = false;
+        for (int64_t c = blockIdx.x; c * sb < a.B; c += gridDim.x)
+            any = any || (tid < sb && c * sb + tid < a.B && is_marked(a.logP[4 * (c * sb + tid)]));
+        if (!__syncthreads_or(any)) return;
+    }
     // [part][c][k]: f pair of the odd row, g pair of the even row before it;
     // k = H: the last even row's g
     T* tab = reinterpret_cast<T*>(smem);
@@ -143,9 +164,10 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
     T* share = res_z + units;                             // [unit][2]
     int* res_e = reinterpret_cast<int*>(share + 2 * units);
     double* larger = reinterpret_cast<double*>(res_e + units);               // [warp][part] (units: a multiple of 4)
-    uint32_t* bits = reinterpret_cast<uint32_t*>(larger + S::NT / 32 * 2);
+    int* low = reinterpret_cast<int*>(larger + S::NT / 32 * 2);              // [unit]: an entry left the range
+    uint32_t* bits = reinterpret_cast<uint32_t*>(low + units);
 
-    bool ok = true;
+    bool ok = true, rare = false;
     double prod[2] = {1.0, 1.0};
     for (int i = tid; i < nu / 2 * D * (H + 1); i += S::NT) {
         const int part = i / (D * (H + 1)), c = i / (H + 1) % D, k = i % (H + 1);
@@ -154,6 +176,7 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
         const float f = k < H ? p[qubit_of<D>(part, c, 2 * k + 1)] : 0.5f;
         ok = ok && g > 0.f && g < 1.f && f > 0.f && f < 1.f;                 // NaN fails
         double top = odds_of(tab + 4 * i + 2, g), f_top = odds_of(tab + 4 * i, f);
+        rare = rare || !(small_rate(g) >= kPairRate) || !(small_rate(f) >= kPairRate);
         if (k < H) top *= f_top;
         if (part) prod[1] *= top;
         else prod[0] *= top;
@@ -169,6 +192,11 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
         larger[(tid >> 5 << 1) + 1] = prod[1];
     }
     const int64_t nchunks = (a.B + sb - 1) / sb;
+    if (__syncthreads_or(rare) && S::kPairs) {
+        for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x)
+            if (tid < sb && c * sb + tid < a.B) a.logP[4 * (c * sb + tid)] = NAN;
+        return;
+    }
     const int unit = tid / S::LANES, lane = tid % S::LANES;
     const int sub = unit / nu, part = unit % nu >> 1, sector = unit & 1;
     const T* ptab = tab + (size_t)part * D * (H + 1) * 4;
@@ -176,7 +204,13 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
     for (int64_t chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
         const int64_t b0 = chunk * sb;
         const int live = (int)(a.B - b0 < sb ? a.B - b0 : sb);
+        bool mine = true;                                 // this thread's syndrome is to be written
+        if constexpr (WIDE) {
+            mine = tid < live && is_marked(a.logP[4 * (b0 + tid)]);
+            if (!__syncthreads_or(mine)) continue;
+        }
         done += live;
+        if (LB > 0 && lane == 0) low[unit] = 0;
         // representative bits: 32 at a time, a lane each, collected by a ballot
         {
             const int wl = tid & 31, nr = nu / 2 * (S::NI / 32);
@@ -258,6 +292,7 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
                     uint32_t toggle = 0;
                     if (j == RB) {
                         uint32_t mx = max_bits(v);
+                        if (min_bits(v) < Range<T>::low) low[unit] = 1;
                         if constexpr (S::LANES >= 32) {
                             mx = __reduce_max_sync(0xffffffffu, mx);
                         } else {
@@ -304,6 +339,7 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
         // the last even row of the last column weights row pair H-1 = register bit RB-1
         T z;
         {
+            if (LB > 0 && min_bits(v) < Range<T>::low) low[unit] = 1;
             T s0 = v[0], s1 = v[R / 2];
 #pragma unroll
             for (int i = 1; i < R / 2; ++i) {
@@ -324,7 +360,12 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
             res_e[unit] = e2;
         }
         __syncthreads();
-        if (tid < live) {
+        bool out = false;                                 // of the range
+        if (LB > 0 && tid < live && mine)
+            for (int s = 0; s < nu; ++s) out = out || low[tid * nu + s];
+        if (out && S::kPairs) {
+            a.logP[4 * (b0 + tid)] = NAN;
+        } else if (tid < live && mine) {
             double larger_m[2] = {1.0, 1.0};              // m 2^e
             int larger_e[2] = {0, 0};
             for (int p = 0; p < nu / 2; ++p) {
@@ -333,7 +374,7 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
             }
             const int64_t b = b0 + tid;
             double lx[2], lz[2];
-            bool bad = false;
+            bool bad = out;
             for (int s = 0; s < 2; ++s) {
                 const double zx = value_of(res_z[tid * nu + s]);
                 bad = bad || !(zx > 0.0) || !(zx < INFINITY);
@@ -370,9 +411,10 @@ __global__ void __launch_bounds__(Shape<H>::NT) xz_kernel(Args a) {
 
 constexpr int kMaxDevices = 64;
 
-template <int H>
-mld_status launch_h(const Args& a, cudaStream_t s) {
-    using S = Shape<H>;
+template <int H, bool WIDE>
+mld_status launch_pass(const Args& a, cudaStream_t s) {
+    using S = Shape<H, WIDE>;
+    const auto kernel = xz_kernel<H, WIDE>;
     const int units = S::NT / S::LANES;
     const size_t smem = shared_bytes<S>(units);
     int dev = 0;
@@ -382,11 +424,11 @@ mld_status launch_h(const Args& a, cudaStream_t s) {
     if (n == 0) {
         int sms = 0, per_sm = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaFuncSetAttribute(xz_kernel<H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)std::max(smem, (size_t)48 * 1024)) != cudaSuccess ||
-            cudaFuncSetAttribute(xz_kernel<H>, cudaFuncAttributePreferredSharedMemoryCarveout,
+            cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xz_kernel<H>, S::NT, smem) != cudaSuccess)
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, S::NT, smem) != cudaSuccess)
             return MLD_ERR_CUDA;
         if (per_sm < 1) return MLD_ERR_UNSUPPORTED;
         n = sms * per_sm;
@@ -395,8 +437,17 @@ mld_status launch_h(const Args& a, cudaStream_t s) {
     const int sb = S::NT / ((a.pz ? 4 : 2) * S::LANES);
     int64_t blocks = (a.B + sb - 1) / sb;
     if (blocks > n) blocks = n;
-    xz_kernel<H><<<(unsigned)blocks, S::NT, smem, s>>>(a);
+    kernel<<<(unsigned)blocks, S::NT, smem, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? MLD_OK : MLD_ERR_CUDA;
+}
+
+template <int H>
+mld_status launch_h(const Args& a, cudaStream_t s) {
+    const mld_status st = launch_pass<H, false>(a, s);
+    if constexpr (Shape<H>::kPairs) {
+        if (st == MLD_OK) return launch_pass<H, true>(a, s);
+    }
+    return st;
 }
 
 mld_status launch(int d, const Args& a, cudaStream_t s) {

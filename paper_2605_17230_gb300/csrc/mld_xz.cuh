@@ -194,13 +194,16 @@ __device__ __forceinline__ void unit_sync(int unit) {
         __syncwarp();
 }
 
-// Entries are kept near the top of the exponent range (between two rescalings
-// they grow by at most 2^H: 1 + odds <= 2 a gate).
+// Entries are kept near the top of the exponent range. Between two rescalings
+// they grow by at most 2^H (1 + odds <= 2 a gate). An operation loses at most
+// a few of the smallest subnormals, 2^14 of them in an entry by the next
+// rescaling; entries of at least 2^-low there keep their accuracy.
 template <typename T>
 struct Range;
 template <>
 struct Range<double> {
     static constexpr int top = 900;
+    static constexpr uint32_t low = (uint32_t)(1023 - 980) << 20;
     static __device__ __forceinline__ double start() { return __hiloint2double((1023 + top) << 20, 0); }
     // bits of the largest entry: its high word, which orders alike
     static __device__ __forceinline__ uint32_t bits(double v) { return (uint32_t)__double2hiint(v); }
@@ -214,6 +217,7 @@ struct Range<double> {
 template <>
 struct Range<Twin> {
     static constexpr int top = gate::kTop;
+    static constexpr uint32_t low = (uint32_t)(127 - 80) << 23;
     static __device__ __forceinline__ Twin start() { return Twin{gate::top_scale(), 0.f}; }
     static __device__ __forceinline__ uint32_t bits(Twin v) { return __float_as_uint(v.hi); }
     static __device__ __forceinline__ float rescale(uint32_t m, int& e2) { return gate::rescale<>(m, e2); }
@@ -225,6 +229,14 @@ __device__ __forceinline__ uint32_t max_bits(const T (&v)[N]) {
     for (int i = 0; i < N; i += 2) m = __vimax3_u32(m, Range<T>::bits(v[i]), Range<T>::bits(v[i + 1]));
     return m;
 }
+template <typename T, int N>
+__device__ __forceinline__ uint32_t min_bits(const T (&v)[N]) {
+    uint32_t m = Range<T>::bits(v[0]);
+#pragma unroll
+    for (int i = 0; i < N; i += 2) m = __vimin3_u32(m, Range<T>::bits(v[i]), Range<T>::bits(v[i + 1]));
+    return m;
+}
+
 // z = m 2^e, m in [sqrt(1/2), sqrt(2)), by its bits (z > 0); e is added.
 __device__ __forceinline__ double mantissa(double z, int& e) {
     if (__double2hiint(z) < 1 << 20) {                    // subnormal

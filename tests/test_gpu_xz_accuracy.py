@@ -1,6 +1,7 @@
-"""FP64 decodes under independent X/Z noise at d >= 15 (pairs of FP32 numbers),
-against the sum over each part's patterns by a column transfer on (d-1)/2 + 1
-bits in extended precision: all four classes.
+"""FP64 decodes under independent X/Z noise at d >= 15 (pairs of FP32 numbers,
+and FP64 where rates leave their range), against the sum over each part's
+patterns by a column transfer on (d-1)/2 + 1 bits in extended precision: all
+four classes, at every rate.
 
 Tolerance: a column's (d-1)/2 gates are each off by 2^-46 (pairs: products and
 sums of 2^-47, weights of 2^-49), so the 2 d (d-1)/2 of a decode are off by at
@@ -88,3 +89,47 @@ def test_uniform_rates(mld, d):
     assert status == 0
     np.testing.assert_allclose(lp, ref, rtol=0, atol=2 * 0.1 * d * d * 2.0 ** -49 + 3 * d * 2.0 ** -47)
     assert np.array_equal(am, np.argmax(lp, axis=1))
+
+
+RATES = ["0.1", "0.01", "1e-4", "1e-6", "1e-8", "1e-12", "mixed", "mostly certain"]
+
+
+@pytest.mark.parametrize("d", [15, 17, 21, 25])
+@pytest.mark.parametrize("rates", RATES)
+def test_every_rate(mld, d, rates):
+    """From typical to dense errors, where entries of a column lie (p)^d below
+    its largest, and with certain errors on half of the qubits."""
+    rng = np.random.default_rng(d)
+    n = d * d
+    if rates == "mixed":
+        px, pz = (10 ** rng.uniform(-8, -0.5, n) for _ in range(2))
+    elif rates == "mostly certain":
+        px, pz = (np.where(rng.random(n) < 0.5, 1e-6, 1 - 1e-6) for _ in range(2))
+    else:
+        px = pz = np.full(n, float(rates))
+    px, pz = px.astype(np.float32), pz.astype(np.float32)
+    syn = _syndromes(d, [0.0, 0.02, 0.1, 0.3, 0.5], rng)
+    ref = _reference(d, px, pz, syn)
+    lp, am, status = _decode(mld, d, px, pz, syn)
+    assert status == 0
+    np.testing.assert_allclose(lp, ref, rtol=1e-15, atol=1e-11)
+    assert np.array_equal(am, np.argmax(lp, axis=1))
+
+
+@pytest.mark.parametrize("d,B", [(15, 37), (17, 9), (25, 3)])
+@pytest.mark.parametrize("bitflip", [False, True])
+def test_marked_among_others(mld, d, B, bitflip):
+    """Dense errors beside typical ones at p = 1e-4 in one batch: only some
+    leave the pairs' range, and each gives the same bits alone."""
+    rng = np.random.default_rng(B)
+    p = np.full(d * d, 1e-4, np.float32)
+    syn = _syndromes(d, rng.choice([0.0, 0.02, 0.5], B), rng)
+    code = mld.Code(d)
+    tp = torch.tensor(p, device="cuda")
+    ts = torch.tensor(syn.view(np.int64), device="cuda")
+    lp, am = code.decode_xz(tp, None if bitflip else tp, ts, mld.MLD_FP64)
+    assert not torch.isnan(lp).any()
+    for b in range(B):
+        one, oam = code.decode_xz(tp, None if bitflip else tp, ts[b:b + 1], mld.MLD_FP64)
+        assert torch.equal(lp[b:b + 1], one) and torch.equal(am[b:b + 1], oam)
+    assert code.status() == 0
