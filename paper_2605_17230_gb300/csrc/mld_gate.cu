@@ -82,9 +82,11 @@ struct ThreadShape {
 };
 
 template <int NB>
-__device__ __forceinline__ float2 finish(float2 (&S)[1 << NB], const float4* w) {
+__device__ __forceinline__ float2 finish(float2 (&S)[1 << NB], const float4* w, int (&e)[2]) {
     // last column from its second row on: halves are l_X = 0, 1; w[0] odd row
-    // (control toggled by l_X), w[1] even row (flip toggled, new bit 0)
+    // (control toggled by l_X), w[1] even row (flip toggled, new bit 0). The
+    // classes part here (one may pay a rate in every row), so each is rescaled
+    // by itself between the row pairs.
     gate_bit<NB, 0>(S, w[0]);
     const float4 v = w[1];
     float2 out[1 << (NB - 2)];
@@ -100,10 +102,17 @@ __device__ __forceinline__ float2 finish(float2 (&S)[1 << NB], const float4* w) 
         }
         out[k] = acc;
     }
-    if constexpr (NB == 2)
+    if constexpr (NB == 2) {
         return out[0];
-    else
-        return finish<NB - 2>(out, w + 2);
+    } else {
+        float2 m = out[0];
+#pragma unroll
+        for (int k = 1; k < (1 << (NB - 2)); ++k) m = make_float2(fmaxf(m.x, out[k].x), fmaxf(m.y, out[k].y));
+        const float2 sc = make_float2(rescale<>(__float_as_uint(m.x), e[0]), rescale<>(__float_as_uint(m.y), e[1]));
+#pragma unroll
+        for (int k = 0; k < (1 << (NB - 2)); ++k) out[k] = mul2(sc, out[k]);
+        return finish<NB - 2>(out, w + 2, e);
+    }
 }
 
 template <int D, bool DEPOL, bool TIES>
@@ -173,7 +182,7 @@ __device__ __forceinline__ void thread_body(const GateArgs& a, const float4* tab
             const auto w = [&](int T) { return weight(0, T + 1, W[0]); };
             Grow<S::NB, 0, decltype(w)>::odd(P, ext, w);
         }
-        float sc = 1.f;
+        float sc = rescale<>(__float_as_uint(max_of(P)), e2);
 #pragma unroll 1
         for (int i = 0; 2 * i + 1 < D - 1; ++i) {
             {
@@ -206,8 +215,9 @@ __device__ __forceinline__ void thread_body(const GateArgs& a, const float4* tab
         for (int j = 0; j < D; ++j) wl[j] = weight(D - 1, j, W[0]);
         wl[0] = make_float4(wl[0].x * sc, wl[0].y * sc, wl[0].z * sc, wl[0].w * sc);
         gate_pair<S::NB>(P, wl[0]);
-        const float2 z = finish<S::NB>(P, wl + 1);
-        const double l0 = ln_scaled(z.x, e2), l1 = ln_scaled(z.y, e2);
+        int e[2] = {e2, e2};
+        const float2 z = finish<S::NB>(P, wl + 1, e);
+        const double l0 = ln_scaled(z.x, e[0]), l1 = ln_scaled(z.y, e[1]);
         const int best = best_of_pair(l0, l1, lz, 0xffffffffu);
         if (live) {
             if ((!(z.x < INFINITY) || !(z.y < INFINITY)) && a.status) atomicOr(a.status, kNumeric);
@@ -480,6 +490,35 @@ __device__ __forceinline__ void lane_body(const GateArgs& a, const float4* table
             v0 = fmaf(u.x, x0, u.z * ox0) + fmaf(u.y, y0, u.w * oy0);
             v1 = fmaf(u.z, x1, u.x * ox1) + fmaf(u.w, y1, u.y * oy1);
         }
+        // the classes have parted on the register side (one may have paid a
+        // rate in every row): each is rescaled by itself
+        int e_0 = e2, e_1 = e2;
+        {
+            uint32_t m0 = __float_as_uint(v0), m1 = __float_as_uint(v1);
+            if constexpr (S::LANES == 16) {
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) {
+                    m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+                    m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+                }
+            } else {
+                m0 = __reduce_max_sync(0xffffffffu, m0);
+                m1 = __reduce_max_sync(0xffffffffu, m1);
+            }
+            if constexpr (S::LANES == 64) {
+                float* x = pair_x + lz * 8;
+                if (wl == 0) {
+                    x[(lane >> 5) * 2] = __uint_as_float(m0);
+                    x[(lane >> 5) * 2 + 1] = __uint_as_float(m1);
+                }
+                unit_sync<D>(lz);
+                m0 = __float_as_uint(fmaxf(x[0], x[2]));
+                m1 = __float_as_uint(fmaxf(x[1], x[3]));
+                unit_sync<D>(lz);
+            }
+            v0 *= rescale<>(m0, e_0);
+            v1 *= rescale<>(m1, e_1);
+        }
         // the lane side: valid where the even positions' lane bits are 0
 #pragma unroll
         for (int t = M & 1; t < M; ++t) {
@@ -513,8 +552,8 @@ __device__ __forceinline__ void lane_body(const GateArgs& a, const float4* table
         if (lane == 0) {
             slot_z[slot * 4 + 2 * lz] = v0;
             slot_z[slot * 4 + 2 * lz + 1] = v1;
-            slot_e[slot * 4 + 2 * lz] = e2;
-            slot_e[slot * 4 + 2 * lz + 1] = e2;
+            slot_e[slot * 4 + 2 * lz] = e_0;
+            slot_e[slot * 4 + 2 * lz + 1] = e_1;
         }
         // logarithms, decisions and stores of up to eight syndromes at a time:
         // one lane per (syndrome, class)
