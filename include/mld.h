@@ -290,8 +290,8 @@ mld_status mld_code_set_truncation_workspace(mld_code* code, int max_bond);
  * boundary MPS of Sec. 3.2.1 discards nothing and is the exact boundary state
  * over one corner column): 0 (default) the column transfer for d <= 13 (the
  * boundary state held densely, d bits, one 2x2 gate per qubit; FP32 for
- * either precision; a syndrome whose two best classes tie up to rounding is
- * decided by the boundary-MPS sweep at d <= 9); 1 always the boundary-MPS
+ * either precision; of a syndrome whose two best classes lie within 1e-5,
+ * ln Z and the decision come from the boundary-MPS sweep at d <= 9); 1 always the boundary-MPS
  * kernel (sites at the exact cut ranks, compile-time plan per d; split-TF32
  * tensor-core products for MLD_MIXED_TF32 at d = 9, 11); 2 as 0 (d = 9, 11,
  * 13). Both give ln Z_l to FP32 accuracy at usual rates. At low ones the
@@ -418,7 +418,7 @@ mld_status mld_measure_fp32_peak(double seconds, double* tflops, int* sm_count);
 
 /* Number of kernel launches one untruncated mld_decode call with an argmax
  * output makes at most for d <= 13 (the column transfer, which checks the
- * noise and takes the decisions, and at d = 9 the pass over tied syndromes;
+ * noise and takes the decisions, and at d <= 9 the pass over tied syndromes;
  * for accounting). */
 int mld_decode_launches(void);
 

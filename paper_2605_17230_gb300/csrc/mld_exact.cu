@@ -33,8 +33,14 @@ bool launch_exact(int d, const ExactArgs& a, cudaStream_t s, int warps_per_block
     return false;
 }
 
-bool launch_decide_ties(const ExactArgs& a, uint8_t* argmax, int precision, int sms, cudaStream_t s) {
-    return exact::launch_ties_d<9>(a, argmax, precision, sms, s);
+bool launch_decide_ties(int d, const ExactArgs& a, uint8_t* argmax, int precision, cudaStream_t s) {
+    switch (d) {
+        case 3: return exact::launch_ties_d<3>(a, argmax, precision, s);
+        case 5: return exact::launch_ties_d<5>(a, argmax, precision, s);
+        case 7: return exact::launch_ties_d<7>(a, argmax, precision, s);
+        case 9: return exact::launch_ties_d<9>(a, argmax, precision, s);
+    }
+    return false;
 }
 
 }  // namespace mld

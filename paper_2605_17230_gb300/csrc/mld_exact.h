@@ -24,7 +24,8 @@ struct ExactArgs {
 int exact_floats_per_warp(int d);
 bool launch_exact(int d, const ExactArgs& a, cudaStream_t s, int warps_per_block, int precision);
 
-// The pass that decides the ties marked in a batch's decisions (d = 9).
-bool launch_decide_ties(const ExactArgs& a, uint8_t* argmax, int precision, int sms, cudaStream_t s);
+// The pass that decides the ties marked in a batch (logP[b][0] NaN; d <= 9);
+// argmax may be nullptr.
+bool launch_decide_ties(int d, const ExactArgs& a, uint8_t* argmax, int precision, cudaStream_t s);
 
 }  // namespace mld

@@ -16,6 +16,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <type_traits>
 #include <utility>
 
@@ -1014,19 +1015,20 @@ __device__ __forceinline__ void decode_unit(const ExactArgs& a, float* ws, int64
     }
 }
 
-// Decides again a syndrome that the column transfer marked: its two best
-// classes are equal up to rounding, as lattice symmetries make them under
-// uniform noise (5 to 18 of 65,536 syndromes at d = 9, p = 0.10; 4% at d = 5,
-// p = 0.19). Which class wins such a tie is a matter of rounding alone, so ln Z
-// and the decision come from this sweep, whichever kernel decodes the rest of
-// the batch. One warp; lane 0 has stored the four values that it compares.
-template <int D, int PREC>
+// Decides again a syndrome that the column transfer marked (logP[b][0] NaN): its
+// two best classes are equal up to rounding, as lattice symmetries make them
+// under uniform noise (5 to 18 of 65,536 syndromes at d = 9, p = 0.10; 4% at
+// d = 5, p = 0.19). Which class wins such a tie is a matter of rounding alone,
+// so ln Z and the decision come from this sweep, whichever kernel decodes the
+// rest of the batch, and whether or not decisions are asked for.
+__device__ __forceinline__ bool is_tie(double l) { return l != l; }
 __device__ __forceinline__ void decide_from(const ExactArgs& a, uint8_t* argmax, int64_t b) {
     int best = 0;
     for (int l = 1; l < 4; ++l)
         if (a.logP[4 * b + l] > a.logP[4 * b + best]) best = l;
     argmax[b] = (uint8_t)best;
 }
+// One warp, in the kernel that found the tie.
 template <int D, int PREC>
 __device__ __noinline__ void decide_tie(const ExactArgs& a, uint8_t* argmax, float* ws, int64_t b, int lane) {
 #pragma unroll 1
@@ -1034,36 +1036,48 @@ __device__ __noinline__ void decide_tie(const ExactArgs& a, uint8_t* argmax, flo
         decode_unit<D, PREC>(a, ws, 2 * b + lz, lane);
         __syncwarp();
     }
-    if (lane == 0) decide_from<D, PREC>(a, argmax, b);
+    if (argmax && lane == 0) decide_from(a, argmax, b);
 }
 
-// The same as a pass over a batch's decisions (bit 7 marks), where the marking
-// kernel has no room for this sweep's state: a block of two warps (l_Z = 0, 1)
-// looks at 128 decisions at a time. The pass lasts one sweep's latency.
+// The same as a pass over a batch: a block lists the ties of its share of the
+// batch, its warps sweep their units, and its threads take the decisions. Ties
+// are few and their sweeps long (15 us alone at d = 7), so a batch is dealt over
+// as many blocks as it fills with a syndrome for each pair of warps.
+template <int D>
+constexpr int kTieWarps = D <= 7 ? 8 : 2;
+template <int D>
+constexpr int kTieBlocksPerSm = D == 3 ? 8 : (D == 5 ? 6 : (D == 7 ? 3 : 5));
 template <int D, int PREC>
-__global__ void __launch_bounds__(64) decide_ties_kernel(ExactArgs a, uint8_t* argmax) {
-    constexpr int FPW = LayoutOf<D>::lay.floats_per_warp;
+__global__ void __launch_bounds__(32 * kTieWarps<D>, PREC == MLD_FP32 ? kTieBlocksPerSm<D> : 1)
+decide_ties_kernel(ExactArgs a, uint8_t* argmax) {
+    constexpr int FPW = LayoutOf<D>::lay.floats_per_warp, NT = 32 * kTieWarps<D>, CAP = 2 * NT;
     extern __shared__ float4 smem4[];
-    const int lz = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* ws = reinterpret_cast<float*>(smem4) + (size_t)lz * FPW;
-    for (int64_t b0 = (int64_t)blockIdx.x * 128; b0 < a.B; b0 += (int64_t)gridDim.x * 128) {
-        int mine = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int64_t b = b0 + 32 * k + lane;
-            mine |= (b < a.B && (argmax[b] & 0x80)) << k;
+    __shared__ int64_t list[CAP];
+    __shared__ int listed;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* ws = reinterpret_cast<float*>(smem4) + (size_t)warp * FPW;
+    int64_t next = (int64_t)blockIdx.x * a.B / gridDim.x;
+    const int64_t end = ((int64_t)blockIdx.x + 1) * a.B / gridDim.x;
+    while (next < end) {
+        if (threadIdx.x == 0) listed = 0;
+        __syncthreads();
+        for (int room = CAP; room >= NT && next < end; next += NT) {
+            const int64_t b = next + threadIdx.x;
+            if (b < end && is_tie(a.logP[4 * b])) list[atomicAdd(&listed, 1)] = b;
+            __syncthreads();
+            room = CAP - listed;
+            __syncthreads();
         }
-        if (!__syncthreads_or(mine)) continue;        // both warps have read the marks
-        for (int k = 0; k < 4; ++k) {
-            unsigned marked = __ballot_sync(0xffffffffu, (mine >> k) & 1);
-            while (marked) {
-                const int64_t b = b0 + 32 * k + __ffs(marked) - 1;
-                marked &= marked - 1;
-                decode_unit<D, PREC>(a, ws, 2 * b + lz, lane);
-                __syncthreads();
-                if (threadIdx.x == 0) decide_from<D, PREC>(a, argmax, b);
-            }
+        const int n = listed;
+#pragma unroll 1
+        for (int u = warp; u < 2 * n; u += kTieWarps<D>) {
+            decode_unit<D, PREC>(a, ws, 2 * list[u >> 1] + (u & 1), lane);
+            __syncwarp();
         }
+        __syncthreads();
+        if (argmax)
+            for (int i = threadIdx.x; i < n; i += NT) decide_from(a, argmax, list[i]);
+        __syncthreads();
     }
 }
 
@@ -1104,21 +1118,38 @@ bool launch_d(const ExactArgs& a, cudaStream_t s, int warps_per_block, int preci
 }
 
 template <int D, int PREC>
-bool launch_ties_dp(const ExactArgs& a, uint8_t* argmax, int sms, cudaStream_t s) {
-    constexpr size_t smem = 2 * (size_t)LayoutOf<D>::lay.floats_per_warp * sizeof(float);
-    static_assert(smem <= 48 * 1024, "two warps' states in a block's default shared memory");
-    int64_t blocks = (a.B + 127) / 128;
-    if (blocks > 4 * (int64_t)sms) blocks = 4 * (int64_t)sms;
-    decide_ties_kernel<D, PREC><<<(unsigned)blocks, 64, smem, s>>>(a, argmax);
+bool launch_ties_dp(const ExactArgs& a, uint8_t* argmax, cudaStream_t s) {
+    constexpr size_t smem = kTieWarps<D> * (size_t)LayoutOf<D>::lay.floats_per_warp * sizeof(float);
+    static_assert(smem <= 48 * 1024, "the warps' states in a block's default shared memory");
+    constexpr int kMaxDevices = 64;
+    static std::atomic<int> resident[kMaxDevices];         // blocks the device holds at once
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+    int n = resident[dev].load(std::memory_order_acquire);
+    if (n == 0) {
+        int sms = 0, per_sm = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaFuncSetAttribute(decide_ties_kernel<D, PREC>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decide_ties_kernel<D, PREC>, 32 * kTieWarps<D>,
+                                                          smem) != cudaSuccess ||
+            per_sm < 1)
+            return false;
+        n = sms * per_sm;
+        resident[dev].store(n, std::memory_order_release);
+    }
+    int64_t blocks = (2 * a.B + kTieWarps<D> - 1) / kTieWarps<D>;
+    if (blocks > n) blocks = n;
+    decide_ties_kernel<D, PREC><<<(unsigned)blocks, 32 * kTieWarps<D>, smem, s>>>(a, argmax);
     return cudaGetLastError() == cudaSuccess;
 }
 
 template <int D>
-bool launch_ties_d(const ExactArgs& a, uint8_t* argmax, int precision, int sms, cudaStream_t s) {
+bool launch_ties_d(const ExactArgs& a, uint8_t* argmax, int precision, cudaStream_t s) {
     if constexpr (kTensorPays<D>) {
-        if (precision == MLD_MIXED_TF32) return launch_ties_dp<D, MLD_MIXED_TF32>(a, argmax, sms, s);
+        if (precision == MLD_MIXED_TF32) return launch_ties_dp<D, MLD_MIXED_TF32>(a, argmax, s);
     }
-    return launch_ties_dp<D, MLD_FP32>(a, argmax, sms, s);
+    return launch_ties_dp<D, MLD_FP32>(a, argmax, s);
 }
 
 }  // namespace exact

@@ -38,7 +38,7 @@ __device__ __forceinline__ const uint64_t* mask_row(const uint64_t* dmask, int d
     return dmask + ((size_t)(r * d + c) * 2 + z) * words;
 }
 
-// Classes within this of the best are a tie: ten times the largest difference
+// Classes within this of the best are a tie: four times the largest difference
 // seen between two kernels' FP32 roundings of one ln Z (2.5e-6 at d = 9).
 constexpr double kTie = 1e-5;
 
@@ -221,12 +221,13 @@ __device__ __forceinline__ void thread_body(const GateArgs& a, const float4* tab
         const int best = best_of_pair(l0, l1, lz, 0xffffffffu);
         if (live) {
             if ((!(z.x < INFINITY) || !(z.y < INFINITY)) && a.status) atomicOr(a.status, kNumeric);
-            a.logP[b * 4 + 2 * lz] = l0;
+            const bool mark = TIES && a.mark_ties && lz == 0 && (best & 0x80);
+            a.logP[b * 4 + 2 * lz] = mark ? (double)NAN : l0;
             a.logP[b * 4 + 2 * lz + 1] = l1;
             if (a.argmax && lz == 0) a.argmax[b] = (uint8_t)(best & 3);
         }
         if constexpr (TIES) {
-            if (a.argmax) {
+            if (!a.mark_ties) {
                 unsigned marked = __ballot_sync(0xffffffffu, live && lz == 0 && (best & 0x80));
                 while (marked) {
                     const int l = __ffs(marked) - 1;
@@ -576,11 +577,11 @@ __device__ __forceinline__ void lane_body(const GateArgs& a, const float4* table
                     }
                 }
                 const unsigned near = __ballot_sync(0xffffffffu, best - l < kTie);      // -inf - -inf compares false
-                const int tie = a.mark_ties && __popc(near >> (gt & 28) & 15u) > 1 ? 0x80 : 0;
+                const bool tie = a.mark_ties && __popc(near >> (gt & 28) & 15u) > 1;
                 const int64_t b0 = b - slot;
                 if (live) {
-                    a.logP[b0 * 4 + gt] = l;
-                    if (a.argmax && (gt & 3) == 0) a.argmax[b0 + (gt >> 2)] = (uint8_t)(at | tie);
+                    a.logP[b0 * 4 + gt] = tie && (gt & 3) == 0 ? (double)NAN : l;
+                    if (a.argmax && (gt & 3) == 0) a.argmax[b0 + (gt >> 2)] = (uint8_t)at;
                 }
             }
             group_sync<D>();
@@ -692,9 +693,16 @@ double gate_flops_per_syndrome(int d) {
     return 2.0 * gate * ((double)d * (d - 2) + 3.0);
 }
 
+// Where ties are decided at d <= 7: inside the kernel for single shots (a second
+// launch takes 3 us more of some 23, and a tie among them 15 to 30 us either
+// way), by the second launch above, where the rest of a warp's sixteen syndromes
+// would wait for each tie (65,536 x 4 shots at d = 7, p = 0.02..0.18: 329 us
+// inside, 266 by the pass; 64 at d = 5, p = 0.10: 52 and 33; start 35).
+constexpr int64_t kTiesInside = 2;
+
 bool launch_gate(int d, const GateArgs& args, const GateTable* table, int warps, cudaStream_t s) {
     GateArgs a = args;
-    a.mark_ties = d == 9 && a.argmax && !table;
+    a.mark_ties = !table && (d == 9 || (d < 9 && a.B > kTiesInside));
     bool ok = false;
     switch (d) {
         case 3: ok = dispatch<3>(a, table, warps, s); break;
@@ -704,10 +712,7 @@ bool launch_gate(int d, const GateArgs& args, const GateTable* table, int warps,
         case 11: ok = dispatch<11>(a, table, warps, s); break;
         case 13: ok = dispatch<13>(a, table, warps, s); break;
     }
-    if (!ok || !a.mark_ties) return ok;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
-    return launch_decide_ties(exact_args(a), a.argmax, a.precision, sm_count(dev), s);
+    return ok && (!a.mark_ties || launch_decide_ties(d, exact_args(a), a.argmax, a.precision, s));
 }
 
 }  // namespace mld

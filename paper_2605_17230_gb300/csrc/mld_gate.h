@@ -15,8 +15,8 @@ struct GateArgs {
     int* status;               // status word (bits 1 << mld_status), or nullptr
     int64_t B;
     int noise_mode;
-    int precision;             // of the sweep that decides ties at d = 9
-    bool mark_ties;            // set by launch_gate
+    int precision;             // of the sweep that decides ties
+    bool mark_ties;            // for a second launch; set by launch_gate
 };
 
 constexpr int kGateMaxTableQubits = 121;
@@ -30,8 +30,9 @@ struct GateTable {
 // Distances with a kernel, its counted flops per syndrome (four classes), and
 // the launch: ln Z, the decision and the noise check in one kernel,
 // asynchronous on s; with a noise table or rates in memory, ties at d <= 9 are
-// decided by the boundary-MPS sweep (a second launch at d = 9). warps: warps per block at d = 9 (0: default). table: the
-// noise table by value in place of a.noise (d <= 11), else nullptr.
+// decided by the boundary-MPS sweep (a second launch, but for single shots at
+// d <= 7). warps: warps per block at d = 9 (0: default). table: the noise table
+// by value in place of a.noise (d <= 11), else nullptr.
 bool gate_supported(int d);
 double gate_flops_per_syndrome(int d);
 bool launch_gate(int d, const GateArgs& a, const GateTable* table, int warps, cudaStream_t s);
