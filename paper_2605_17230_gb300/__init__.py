@@ -154,13 +154,15 @@ def _ptr(t):
 def _stream(stream):
     """The cudaStream_t to enqueue on: the given one, or torch's current stream
     of the current device, read as the raw handle (constructing the Stream
-    object takes 2.9 us of a 17 us call)."""
+    object takes 2.9 us of a 17 us call). The two functions that give the handle
+    are torch's own and not public: a torch without them takes the long way."""
     if stream is not None:
         return int(stream)
     import torch
-    if not torch.cuda.is_initialized():
+    raw, device = (getattr(torch._C, f, None) for f in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+    if raw is None or device is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return raw(device())
 
 
 def mld_decode(code, noise, noise_mode, syndromes, B, chi, precision, logP, argmax=None, stream=None):
