@@ -22,21 +22,24 @@
 // gradient that they add up to, and the unit adds nothing from there on
 // (MLD_ERR_NUMERIC).
 //
-// Accuracy: each sum is divided by the Z of the whole sweep (the classes' sum
-// may cancel, so no column's own overlap can take its place): a single shot's
-// gradient is off by 1 to 1.6 times (3.5 times at d = 11 where one path
-// dominates) the 1e-7 to 5e-7 of its largest entry that a sweep per class with
-// each column's own overlap has.
+// Accuracy: a gate's weighted sums add up to the upstream gradients of the two
+// classes, up to the roundings of the states between the gate and Z. The first
+// gate of each side of a column measures the ratio (in FP32 pairs) and the
+// sums of that side are corrected by it, unless the two gradients cancel by
+// half. Against 64 bits, batch gradient of an unlabelled loss, 512 shots: d = 3
+// 3.4e-8 (without 9.2e-8, a sweep per class divided by each column's own
+// overlap 4.4e-8), d = 5 2.8e-8 (8.9e-8, 4.9e-8), d = 7 4.0e-8 (8.8e-8, 5.0e-8),
+// d = 9 4.3e-8 (1.2e-7, 8.1e-8).
 //
 // Bound: at d <= 9 issue and shared memory (50% of the issue slots, 62% of the
 // shared-memory cycles at d = 7: state loads, exchanges, the sums over lanes);
 // at d = 11 the fetching of its own straight-line program (93 KB) by five
 // resident warps an SM. Measured on GB300, against one block per (syndrome,
-// class) with its states in shared memory: d = 7, 65,536 syndromes 0.56 ms
-// (6.1); d = 9, 16,384 syndromes 0.79 ms (8.6; 0.72 without the rescaling of
-// the adjoint state); d = 11, 2,049 syndromes 1.55 ms (7.4; 1.5). A column as a
-// list of operations run by an interpreter (one copy of each gate's code) was
-// slower: 0.92, 1.18, 1.90 ms.
+// class) with its states in shared memory: d = 7, 65,536 syndromes 0.63 ms
+// (6.1; 0.56 without the correction); d = 9, 16,384 syndromes 0.87 ms (8.6;
+// 0.72 without it and the rescaling of the adjoint state); d = 11, 2,049
+// syndromes 1.63 ms (7.4; 1.5). A column as a list of operations run by an
+// interpreter (one copy of each gate's code) was slower: 0.92, 1.18, 1.90 ms.
 //
 // Gradients are summed per unit slot in FP64 in a fixed order, the slots by a
 // second kernel: reruns give the same bits.
@@ -48,11 +51,13 @@
 #include "mld_gate.cuh"
 #include "mld_grad.h"
 #include "mld_internal.h"
+#include "mld_xz.cuh"
 
 namespace mld {
 namespace {
 
 using namespace gate;
+using xz::Twin;
 
 // Tops of the states and of the adjoint states (a class's paths need the range
 // below both): a weight sum adds up to 2^d products of the two, below
@@ -102,6 +107,12 @@ __device__ __forceinline__ float scaled(float x, int e) {
     const int bits = __float_as_int(x), at = (bits >> 23) & 0xff, to = at + e;
     if (at == 0 || to <= 0) return 0.f;
     return to < 0xff ? __int_as_float((bits & ~(0xff << 23)) | to << 23) : copysignf(INFINITY, x);
+}
+
+// a + b of either sign, to FP32 pairs' accuracy of the larger.
+__device__ __forceinline__ Twin add_twins(Twin a, Twin b) {
+    const float s = __fadd_rn(a.hi, b.hi);
+    return xz::renormal(s, __fadd_rn(xz::sum_error(a.hi, b.hi, s), __fadd_rn(a.lo, b.lo)));
 }
 
 template <int M>
@@ -254,8 +265,10 @@ struct Lane {
     // a factor of those of step M+1 and of all before it (early), not of G.
     struct Factors {
         double late, early;
-        float unit, want, slack;    // what a gate's weighted sums times (unit 2^e) come to, and by how much they may miss it
+        Twin unit, want;            // what a gate's weighted sums times (unit 2^e) come to
+        float slack;                // by how much they may miss it
         int e_late, e_early;
+        float drift;                // what they miss, of them
         bool lost;
     };
     // Step J backwards: P is the state before it.
@@ -289,19 +302,34 @@ struct Lane {
         }
         const int r = grad_row(D, c, J), q = r * D + c;
         const uint32_t e = (w >> (2 * J)) & 3;
-        // (the column's first gate: its sums have to give what the unit adds)
-        const auto check = [&](float t) {
+        // (the first gate of each side: its weighted sums have to give what the
+        // unit adds; the ratio takes the roundings between here and Z out)
+        const auto check = [&](float a, float b, float a2 = 0.f, float b2 = 0.f) {
+            const auto product = [](float x, float w) {
+                const float p = __fmul_rn(x, w);
+                return Twin{p, __fmaf_rn(x, w, -p)};
+            };
+            Twin t = product(a, b);
+            if (M == 1) t = xz::plus(t, product(a2, b2));
 #pragma unroll
-            for (int o = 1; o < S::LANES && o < 4; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            t = scaled(__shfl_sync(0xffffffffu, t, 0, S::LANES), J > M + 1 ? by.e_late : by.e_early) * by.unit;
-            by.lost = fabsf(t - by.want) > by.slack;
-            if (by.lost) by.late = by.early = 0.0;
+            for (int o = 1; o < S::LANES && o < 4; o <<= 1) t = xz::plus(t, xz::shuffled(t, o));
+            const int e = J > M + 1 ? by.e_late : by.e_early;
+            t.hi = scaled(__shfl_sync(0xffffffffu, t.hi, 0, S::LANES), e);
+            t.lo = scaled(__shfl_sync(0xffffffffu, t.lo, 0, S::LANES), e);
+            t = xz::times(t, by.unit);
+            const float miss = (by.want.hi - t.hi) + (by.want.lo - t.lo);
+            if (fabsf(miss) > by.slack) {
+                by.lost = true;
+                by.late = by.early = 0.0;
+            }
+            by.drift = fabsf(miss) <= by.slack && fabsf(by.want.hi) > 4.f * by.slack ? miss / t.hi : 0.f;
         };
-        if constexpr (J == D - 1 && M == 1) check((lane & 1) ? fmaf(v0, v.z, v1 * v.w) : fmaf(v0, v.x, v1 * v.y));
+        const float4 y = J == M && bit(0) ? make_float4(v.y, v.x, v.w, v.z) : v;      // as the sums: without the lane's share
+        if constexpr ((J == D - 1 || J == M) && M == 1) check(v0, (lane & 1) ? y.z : y.x, v1, (lane & 1) ? y.w : y.y);
         const auto add = [&](int f, int cc, float x) {
             const int ff = f ^ (int)(e >> 1), c2 = cc ^ (int)(e & 1);
             const int xx = (r & 1) ? c2 : ff, zz = (r & 1) ? ff : c2;
-            acc[4 * q + (xx ? (zz ? 2 : 1) : (zz ? 3 : 0))] += (double)x * (J > M + 1 ? by.late : by.early);
+            acc[4 * q + (xx ? (zz ? 2 : 1) : (zz ? 3 : 0))] += (double)fmaf(x, by.drift, x) * (J > M + 1 ? by.late : by.early);
         };
         if constexpr (M == 1) {
             add(lane & 1, 0, v0);
@@ -311,8 +339,8 @@ struct Lane {
             float x = (up ? v1 : v0) + __shfl_xor_sync(0xffffffffu, up ? v0 : v1, 2);
 #pragma unroll
             for (int o = 4; o < S::LANES; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if constexpr (J == D - 1)
-                check(lane < 4 ? x * ((lane & 1) ? ((lane & 2) ? v.w : v.z) : ((lane & 2) ? v.y : v.x)) : 0.f);
+            if constexpr (J == D - 1 || J == M)
+                check(x, lane < 4 ? ((lane & 1) ? ((lane & 2) ? y.w : y.z) : ((lane & 2) ? y.y : y.x)) : 0.f);
             if (lane < 4) add(lane & 1, lane >> 1, x);
         }
     }
@@ -329,16 +357,17 @@ struct Lane {
         }
     }
     // Column c backwards: G after it -> G before it; factor 2^ge G is the
-    // derivative of the loss by the state (unit is the same in FP32, with the
+    // derivative of the loss by the state (unit is the same factor, with the
     // upstream gradients want, on a common scale). Returns whether the range
     // was lost.
     __device__ __forceinline__ bool back_column(float2 (&G)[1 << M], int c, uint32_t w, int slot, double factor, int& ge,
-                                                float unit, float want, float slack) const {
+                                                Twin unit, Twin want, float slack) const {
         const float sc = scale[slot];
         Factors by;
         by.unit = unit;
         by.want = want;
         by.slack = slack;
+        by.lost = false;
         by.e_late = ge;
         by.late = scaled(factor, ge);
         ge += (int)(__float_as_uint(sc) >> 23) - 127;
@@ -505,10 +534,11 @@ grad_gate_kernel(GradDenseArgs g) {
         float2* second = first - S::STATE;               // the last column's start, read by then
         double c0 = ok0 ? u0 / (double)z[0] : 0.0, c1 = ok1 ? u1 / (double)z[1] : 0.0;
         const int top = 1023 - max(ok0 ? (__double2hiint(u0) >> 20) & 0x7ff : 0, ok1 ? (__double2hiint(u1) >> 20) & 0x7ff : 0);
-        float want0 = ok0 ? (float)scaled(u0, top) : 0.f, want1 = ok1 ? (float)scaled(u1, top) : 0.f;
-        const float slack = 0.125f * (fabsf(want0) + fabsf(want1));
+        Twin want0 = xz::make<Twin>(ok0 ? scaled(u0, top) : 0.0), want1 = xz::make<Twin>(ok1 ? scaled(u1, top) : 0.0);
+        const float slack = 0.125f * (fabsf(want0.hi) + fabsf(want1.hi));
         double factor = 0.0;
-        float per = 0.f, want = 0.f;
+        const Twin none{0.f, 0.f};
+        Twin per = none, want = none;
         bool apart = false, lost = false;
         int ge = 0, ge0 = 0, ge1 = 0, passes = 1;
 #pragma unroll 1
@@ -530,8 +560,9 @@ grad_gate_kernel(GradDenseArgs g) {
                         share = pass || apart ? 0.f : (float)ratio;
                     }
                     factor = pass && !apart ? 0.0 : (one ? c1 : c0);
-                    per = (float)scaled(factor, top);
-                    want = pass && !apart ? 0.f : (step == 2 && !apart ? want0 + want1 : (one ? want1 : want0));
+                    per = xz::make<Twin>(scaled(factor, top));
+                    want = pass && !apart ? none : (one ? want1 : want0);
+                    if (step == 2 && pass == 0 && !apart) want = add_twins(want0, want1);
                     ge = step < 2 ? -kAdjointTop : (one ? ge1 : ge0);
                     if (step < 2) {
                         end_state(G, __uint_as_float((uint32_t)(127 + kAdjointTop) << 23));
@@ -545,8 +576,11 @@ grad_gate_kernel(GradDenseArgs g) {
                 if (L.back_column(G, c, L.word(c, step == 1), step == 1 ? D : c, factor, ge, per, want, slack)) {
                     lost = true;
                     factor = 0.0;
-                    per = want = 0.f;
-                    if (step < 2) (step ? c1 : c0) = (step ? want1 : want0) = 0.f;
+                    per = want = none;
+                    if (step < 2) {
+                        (step ? c1 : c0) = 0.0;
+                        (step ? want1 : want0) = none;
+                    }
                 }
                 if (step < 2) {
                     store_state<M>(G, step ? second : first, lane);

@@ -84,3 +84,23 @@ def test_rare_syndromes(mld, d, name, columns):
         dn, status = _grad(mld, d, noise, syn[b:b + 1], up[b:b + 1])
         assert status == 0
         np.testing.assert_allclose(dn, ref, rtol=2e-5, atol=2e-5 * np.abs(ref).max(), err_msg=str(b))
+
+
+@pytest.mark.parametrize("d", [3, 5, 7, 9])
+def test_batch_gradient_against_64_bits(mld, d):
+    """The marginal likelihood's gradient over a batch. A gate's sums are put
+    on the overlap of the first gate on its side of the column, so at most
+    (d+1)/2 gates of two roundings each separate them, on either state:
+    sqrt(2 (d+1)) 2^-25 / sqrt(3) = 8e-8 a shot at d = 9, in part averaged over
+    the batch: half an ulp, 2^-24, of the gradient's norm."""
+    n, B = d * d, 512
+    noise = synth.lognormal_biased(n, seed=d).astype(np.float32)
+    syn = synth.syndromes_of(d, synth.sample_errors(d, noise, B, seed=1))
+    lz, g = oracle.coset_dlogz(d, noise.astype(np.float64), oracle.representatives(d, syn).reshape(-1, n))
+    lz = lz.reshape(B, 4)
+    post = np.exp(lz - lz.max(axis=1, keepdims=True))
+    up = -post / post.sum(axis=1, keepdims=True) / B
+    ref = np.einsum("bl,blqp->qp", up, g.reshape(B, 4, n, 4))
+    dn, status = _grad(mld, d, noise, syn, up)
+    assert status == 0
+    assert np.linalg.norm(dn - ref) <= 2.0 ** -24 * np.linalg.norm(ref)
