@@ -44,8 +44,8 @@ TF32_PER_BF16 = 1.1 / 2.25          # nominal dense TF32 / BF16 tensor rates of 
 # DRAM bytes per syndrome of the decode kernel (dram__bytes_read.sum + write.sum of one ncu
 # capture of 8,192 syndromes of the headline kernel), valid only for the kernel sources they
 # were taken on: any change to them makes the traffic unknown (null).
-TRAFFIC_SOURCES_SHA = "b992a96b56cd3cbb"
-TRAFFIC_BYTES_PER_SYNDROME = {0: 187.328e3 / 8192, 2: 187.328e3 / 8192}
+TRAFFIC_SOURCES_SHA = "5c51c4d88ccc9b81"
+TRAFFIC_BYTES_PER_SYNDROME = {0: 188.224e3 / 8192, 2: 188.224e3 / 8192}
 # sources of the headline kernel (gate_decode_kernel<9, *>)
 TRAFFIC_SOURCES = ("mld_gate.cuh", "mld_gate.h", "mld_gate.cu")
 

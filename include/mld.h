@@ -67,9 +67,9 @@ typedef enum {
                                   products run at d = 9 and 11, where they are
                                   faster; at other d the FP32 products run
                                   (same or better accuracy) */
-    MLD_FP64 = 3               /* complex FP64 elimination; mld_decode_xz
-                                  only (other entry points return
-                                  MLD_ERR_INVALID_ARG) */
+    MLD_FP64 = 3               /* the parts' column transfer at FP64 accuracy;
+                                  mld_decode_xz only (other entry points
+                                  return MLD_ERR_INVALID_ARG) */
 } mld_precision;
 
 typedef enum {

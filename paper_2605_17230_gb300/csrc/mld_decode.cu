@@ -905,7 +905,7 @@ mld_status decode_truncated(mld_code* C, const mld::Plan& P, const mld::SiteStep
     const int* last_count = reinterpret_cast<const int*>(ctl + 16);
     if (pass2) {
         ta.caps = mld::kTruncLarge;
-        ta.arena = mld::kTruncArenas[2];       // few and heavy units on one block per 4 SMs
+        ta.arena = mld::kTruncArenas[2];       // few and heavy units, one per SM
         ta.next_unit = reinterpret_cast<unsigned long long*>(ctl + 8);
         ta.in_list = C->d_ovf;
         ta.in_count = reinterpret_cast<const int*>(ctl + 16);

@@ -1,7 +1,7 @@
 // Untruncated decode by the column transfer (mld_gate.cuh): d = 3, 5, 7 with
 // one thread per (syndrome, l_Z), d = 9, 11, 13 with the state spread over 16,
 // 32 or 64 lanes. All four classes, the decision and the check of the noise
-// in one launch.
+// in one launch; a second one over ties at d <= 9.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

@@ -165,7 +165,8 @@ struct Grow {
 
 // ln z + e ln 2 for z >= 0. ln of the mantissa m in [sqrt(1/2), sqrt(2)) from
 // the series of 2 atanh((m-1)/(m+1)), the quotient to twice FP32 precision, so
-// that the error stays below 1e-9 (an FP64 log is some 25 instructions of a
+// that the error stays below 2e-9 (1.8e-9 over all mantissas, the operations
+// run on the host; an FP64 log is some 25 instructions of a
 // pipe with 1/64 of the FP32 rate: at d = 5 it would cost more than the sweep).
 __device__ __forceinline__ double ln_scaled(float z, int e) {
     if (!(z > 0.f)) return -INFINITY;
