@@ -296,8 +296,9 @@ mld_status mld_code_set_truncation_workspace(mld_code* code, int max_bond);
  * tensor-core products for MLD_MIXED_TF32 at d = 9, 11); 2 as 0 (d = 9, 11,
  * 13). Both give ln Z_l to FP32 accuracy at usual rates. At low ones the
  * column transfer keeps it while (p/3)^d, the smallest rate of a string, is
- * above 2^-220 (p = 1e-9 at d = 7, 2e-7 at d = 9, 3e-5 at d = 13); below, the
- * less likely classes lose strings, and at last become -inf. The boundary MPS
+ * above 2^-220 (p = 1e-9 at d = 7, 2e-7 at d = 9, 3e-5 at d = 13; under Y
+ * errors alone a string has d^2 of them); below, the less likely classes lose
+ * strings, and at last become -inf. The boundary MPS
  * loses accuracy earlier (0.008 at d = 7, p = 1e-6). MLD_ERR_INVALID_ARG for
  * other values, MLD_ERR_UNSUPPORTED for 2 at other d. Host only. */
 mld_status mld_code_set_exact_kernel(mld_code* code, int which);

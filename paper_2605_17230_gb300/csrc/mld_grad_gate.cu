@@ -25,20 +25,24 @@
 // Accuracy: a gate's weighted sums add up to the upstream gradients of the two
 // classes, up to the roundings of the states between the gate and Z. The first
 // gate of each side of a column measures the ratio (in FP32 pairs) and the
-// sums of that side are corrected by it, unless the two gradients cancel by
-// half. Against 64 bits, batch gradient of an unlabelled loss, 512 shots: d = 3
-// 3.4e-8 (without 9.2e-8, a sweep per class divided by each column's own
-// overlap 4.4e-8), d = 5 2.8e-8 (8.9e-8, 4.9e-8), d = 7 4.0e-8 (8.8e-8, 5.0e-8),
-// d = 9 4.3e-8 (1.2e-7, 8.1e-8).
+// sums of that side are corrected by it. Of classes whose gradients oppose each
+// other by more than a twentieth the common ratio would multiply what sets
+// their own apart, so they are swept back one after the other. Against 64 bits,
+// batch gradient of an unlabelled loss, 512 shots: d = 3 3.4e-8 (without 9.2e-8,
+// a sweep per class divided by each column's own overlap 4.4e-8), d = 5 2.8e-8
+// (8.9e-8, 4.9e-8), d = 7 4.0e-8 (8.8e-8, 5.0e-8), d = 9 4.3e-8 (1.2e-7, 8.1e-8);
+// single shots with gradients 1, -1 of two classes, of their terms: d = 7 8.4e-8
+// (1.8e-7, 1.1e-7), d = 9 1.1e-7 (2.4e-7, 1.3e-7).
 //
 // Bound: at d <= 9 issue and shared memory (50% of the issue slots, 62% of the
 // shared-memory cycles at d = 7: state loads, exchanges, the sums over lanes);
 // at d = 11 the fetching of its own straight-line program (93 KB) by five
 // resident warps an SM. Measured on GB300, against one block per (syndrome,
 // class) with its states in shared memory: d = 7, 65,536 syndromes 0.63 ms
-// (6.1; 0.56 without the correction); d = 9, 16,384 syndromes 0.87 ms (8.6;
-// 0.72 without it and the rescaling of the adjoint state); d = 11, 2,049
-// syndromes 1.63 ms (7.4; 1.5). A column as a list of operations run by an
+// (6.1; 0.56 without the correction; 1.0 where all units hold opposed classes);
+// d = 9, 16,384 syndromes 0.87 ms (8.6; 0.72 without it and the rescaling of the
+// adjoint state; 1.47 opposed); d = 11, 2,049 syndromes 1.0 ms (7.4; 1.9
+// opposed). A column as a list of operations run by an
 // interpreter (one copy of each gate's code) was slower: 0.92, 1.18, 1.90 ms.
 //
 // Gradients are summed per unit slot in FP64 in a fixed order, the slots by a
@@ -64,8 +68,10 @@ using xz::Twin;
 // 2^(54 + 1 + 54 + 1 + 11).
 constexpr int kGradTop = 54, kAdjointTop = 54;
 // Classes whose adjoint states at the start of the last column differ by more
-// than this are swept back one at a time (they would not fit one range).
+// than this are swept back one at a time (they would not fit one range), and
+// so are those whose gradients add up to less than this part of their moduli.
 constexpr double kApart = 8.673617379884035e-19;        // 2^-60
+constexpr float kOpposed = 0.9f;
 
 template <int D>
 struct GradLanes {
@@ -266,7 +272,7 @@ struct Lane {
     struct Factors {
         double late, early;
         Twin unit, want;            // what a gate's weighted sums times (unit 2^e) come to
-        float slack;                // by how much they may miss it
+        float slack, trust;         // by how much they may miss it; and to be corrected
         int e_late, e_early;
         float drift;                // what they miss, of them
         bool lost;
@@ -322,7 +328,7 @@ struct Lane {
                 by.lost = true;
                 by.late = by.early = 0.0;
             }
-            by.drift = fabsf(miss) <= by.slack && fabsf(by.want.hi) > 4.f * by.slack ? miss / t.hi : 0.f;
+            by.drift = by.trust > 0.f && fabsf(miss) <= by.trust ? miss / t.hi : 0.f;
         };
         const float4 y = J == M && bit(0) ? make_float4(v.y, v.x, v.w, v.z) : v;      // as the sums: without the lane's share
         if constexpr ((J == D - 1 || J == M) && M == 1) check(v0, (lane & 1) ? y.z : y.x, v1, (lane & 1) ? y.w : y.y);
@@ -361,12 +367,13 @@ struct Lane {
     // upstream gradients want, on a common scale). Returns whether the range
     // was lost.
     __device__ __forceinline__ bool back_column(float2 (&G)[1 << M], int c, uint32_t w, int slot, double factor, int& ge,
-                                                Twin unit, Twin want, float slack) const {
+                                                Twin unit, Twin want, float slack, float trust) const {
         const float sc = scale[slot];
         Factors by;
         by.unit = unit;
         by.want = want;
         by.slack = slack;
+        by.trust = trust;
         by.lost = false;
         by.e_late = ge;
         by.late = scaled(factor, ge);
@@ -535,10 +542,11 @@ grad_gate_kernel(GradDenseArgs g) {
         double c0 = ok0 ? u0 / (double)z[0] : 0.0, c1 = ok1 ? u1 / (double)z[1] : 0.0;
         const int top = 1023 - max(ok0 ? (__double2hiint(u0) >> 20) & 0x7ff : 0, ok1 ? (__double2hiint(u1) >> 20) & 0x7ff : 0);
         Twin want0 = xz::make<Twin>(ok0 ? scaled(u0, top) : 0.0), want1 = xz::make<Twin>(ok1 ? scaled(u1, top) : 0.0);
-        const float slack = 0.125f * (fabsf(want0.hi) + fabsf(want1.hi));
+        const float moduli = fabsf(want0.hi) + fabsf(want1.hi), slack = 0.125f * moduli;
         double factor = 0.0;
         const Twin none{0.f, 0.f};
         Twin per = none, want = none;
+        float trust = 0.f;
         bool apart = false, lost = false;
         int ge = 0, ge0 = 0, ge1 = 0, passes = 1;
 #pragma unroll 1
@@ -554,7 +562,7 @@ grad_gate_kernel(GradDenseArgs g) {
                         one = fabs(scaled(c1, ge1 - ge0)) > fabs(c0);
                         const double small = one ? scaled(c0, ge0 - ge1) : scaled(c1, ge1 - ge0), big = one ? c1 : c0;
                         const double ratio = small == 0.0 ? 0.0 : small / big;
-                        apart = small != 0.0 && fabs(ratio) < kApart;
+                        apart = small != 0.0 && (fabs(ratio) < kApart || fabsf(want0.hi + want1.hi) < kOpposed * moduli);
                         if (pass == 0) passes = __any_sync(0xffffffffu, apart) ? 2 : 1;
                         if (pass == 1) one = !one;
                         share = pass || apart ? 0.f : (float)ratio;
@@ -563,6 +571,7 @@ grad_gate_kernel(GradDenseArgs g) {
                     per = xz::make<Twin>(scaled(factor, top));
                     want = pass && !apart ? none : (one ? want1 : want0);
                     if (step == 2 && pass == 0 && !apart) want = add_twins(want0, want1);
+                    trust = 0.125f * fabsf(want.hi);
                     ge = step < 2 ? -kAdjointTop : (one ? ge1 : ge0);
                     if (step < 2) {
                         end_state(G, __uint_as_float((uint32_t)(127 + kAdjointTop) << 23));
@@ -573,10 +582,11 @@ grad_gate_kernel(GradDenseArgs g) {
                             G[k] = fma2(dup(share), h[(k << M) + lane], g[(k << M) + lane]);
                     }
                 }
-                if (L.back_column(G, c, L.word(c, step == 1), step == 1 ? D : c, factor, ge, per, want, slack)) {
+                if (L.back_column(G, c, L.word(c, step == 1), step == 1 ? D : c, factor, ge, per, want, slack, trust)) {
                     lost = true;
                     factor = 0.0;
                     per = want = none;
+                    trust = 0.f;
                     if (step < 2) {
                         (step ? c1 : c0) = 0.0;
                         (step ? want1 : want0) = none;
