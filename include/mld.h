@@ -235,17 +235,16 @@ mld_status mld_autotune(const mld_code* code, int chi, int precision, int64_t sa
  * boundary states are kept as their entries (the right states are carried
  * back through each column by the transposed factors): in registers for
  * d <= 11; at d = 13 the states inside a column (128 KB each) live in a device
- * workspace of about 1.7 MB per resident block. The left
- * state at every column boundary is stored by the forward pass (a
- * checkpoint per column) and the states inside a column are recomputed from
- * it during the backward pass. FP32 contraction, FP64
- * accumulation in a fixed order, so reruns give the same bits. Entries keep
- * FP32 accuracy down to 2^-180 of a state's largest (d <= 11). A syndrome with
- * a class whose paths lie further below (rates under 1e-5 and errors all over
- * the patch) loses them: where its gradients would be off by an eighth, it adds
- * nothing from that column on and MLD_ERR_NUMERIC is set in the status word. Asynchronous
- * on stream; uses a device workspace owned by the code object (not reentrant
- * per code). */
+ * workspace of about 1.7 MB per resident block. The left state at every
+ * column boundary is stored by the forward pass (a checkpoint per column) and
+ * the states inside a column are recomputed from it during the backward pass.
+ * FP32 contraction, FP64 accumulation in a fixed order, so reruns give the
+ * same bits. Entries keep FP32 accuracy down to 2^-180 of a state's largest
+ * (d <= 11). A syndrome with a class whose paths lie further below (rates
+ * under 1e-5 and errors all over the patch) loses them: where its gradients
+ * would be off by an eighth, it adds nothing from that column on and
+ * MLD_ERR_NUMERIC is set in the status word. Asynchronous on stream; uses a
+ * device workspace owned by the code object (not reentrant per code). */
 mld_status mld_decode_grad(const mld_code* code, const float* noise, const uint64_t* syndromes, int64_t B,
                            int chi, const double* dlogP, double* logP, double* dnoise, void* stream);
 
@@ -291,15 +290,14 @@ mld_status mld_code_set_truncation_workspace(mld_code* code, int max_bond);
  * over one corner column): 0 (default) the column transfer for d <= 13 (the
  * boundary state held densely, d bits, one 2x2 gate per qubit; FP32 for
  * either precision; of a syndrome whose two best classes lie within 1e-5,
- * ln Z and the decision come from the boundary-MPS sweep at d <= 9); 1 always the boundary-MPS
- * kernel (sites at the exact cut ranks, compile-time plan per d; split-TF32
- * tensor-core products for MLD_MIXED_TF32 at d = 9, 11); 2 as 0 (d = 9, 11,
- * 13). Both give ln Z_l to FP32 accuracy at usual rates. At low ones the
+ * ln Z and the decision come from the boundary-MPS sweep at d <= 9); 1 always
+ * the boundary-MPS kernel (sites at the exact cut ranks, compile-time plan per
+ * d; split-TF32 tensor-core products for MLD_MIXED_TF32 at d = 9, 11); 2 as 0
+ * (d = 9, 11, 13). Both give ln Z_l to FP32 accuracy at usual rates. At low ones the
  * column transfer keeps it while (p/3)^d, the smallest rate of a string, is
  * above 2^-220 (p = 1e-9 at d = 7, 2e-7 at d = 9, 3e-5 at d = 13; under Y
  * errors alone a string has d^2 of them); below, the less likely classes lose
- * strings, and at last become -inf. The boundary MPS
- * loses accuracy earlier (0.008 at d = 7, p = 1e-6). MLD_ERR_INVALID_ARG for
+ * strings, and at last become -inf. The boundary MPS loses accuracy earlier (0.008 at d = 7, p = 1e-6). MLD_ERR_INVALID_ARG for
  * other values, MLD_ERR_UNSUPPORTED for 2 at other d. Host only. */
 mld_status mld_code_set_exact_kernel(mld_code* code, int which);
 

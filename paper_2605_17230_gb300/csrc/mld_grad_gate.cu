@@ -115,12 +115,6 @@ __device__ __forceinline__ float scaled(float x, int e) {
     return to < 0xff ? __int_as_float((bits & ~(0xff << 23)) | to << 23) : copysignf(INFINITY, x);
 }
 
-// a + b of either sign, to FP32 pairs' accuracy of the larger.
-__device__ __forceinline__ Twin add_twins(Twin a, Twin b) {
-    const float s = __fadd_rn(a.hi, b.hi);
-    return xz::renormal(s, __fadd_rn(xz::sum_error(a.hi, b.hi, s), __fadd_rn(a.lo, b.lo)));
-}
-
 template <int M>
 __device__ __forceinline__ void load_state(float2 (&P)[1 << M], const float2* s, int lane) {
 #pragma unroll
@@ -570,7 +564,7 @@ grad_gate_kernel(GradDenseArgs g) {
                     factor = pass && !apart ? 0.0 : (one ? c1 : c0);
                     per = xz::make<Twin>(scaled(factor, top));
                     want = pass && !apart ? none : (one ? want1 : want0);
-                    if (step == 2 && pass == 0 && !apart) want = add_twins(want0, want1);
+                    if (step == 2 && pass == 0 && !apart) want = xz::plus(want0, want1);
                     trust = 0.125f * fabsf(want.hi);
                     ge = step < 2 ? -kAdjointTop : (one ? ge1 : ge0);
                     if (step < 2) {

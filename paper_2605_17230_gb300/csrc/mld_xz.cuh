@@ -11,8 +11,8 @@
 namespace mld {
 namespace xz {
 
-// Twice FP32: hi + lo, |lo| <= ulp(hi)/2. Products and sums of non-negative
-// numbers only, so nothing cancels.
+// Twice FP32: hi + lo, |lo| <= ulp(hi)/2. The transfer has products and sums of
+// non-negative numbers only, so nothing cancels.
 struct Twin {
     float hi, lo;
 };
